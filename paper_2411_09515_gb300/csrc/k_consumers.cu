@@ -345,90 +345,181 @@ __global__ void k_scatter_list(const int32_t* idx, const int32_t* n_kept, int64_
 
 constexpr int kPeakThreads = 256;
 constexpr int kPeakChunk = 256;          // kept entries per flag chunk (8 flag words)
-constexpr int kPeakCtasPerFrame = 64;
-constexpr int kPeakList = 4096;         // peaks a record CTA lists in shared memory at once
+constexpr int kPeakList = 2048;          // peaks a record CTA lists in shared memory at once
+constexpr int kPeakCtas = 152 * 8;       // CTAs wanted of either peak kernel (8 of 256 threads fit a multiprocessor)
 
-__device__ __forceinline__ bool is_kept(const uint32_t* bm, int64_t j) { return (bm[j >> 5] >> (j & 31)) & 1u; }
-
-// Is kept pixel i a peak (Section 4)? At least min_count kept pixels in the
-// patch, and i the maximum of the patch's valid pixels (ties: lowest index).
-// (the pixel's own value is loaded only once the bitmap has shown enough
-// kept pixels: most kept pixels are isolated and fail on the count alone)
-template <int DT, bool NORM>
-__device__ __forceinline__ bool peak_test(const PixArgs& p, const void* frame, int64_t f, const uint32_t* bm, int64_t i,
-                                          int h, int32_t min_count) {
-  const int r0 = (int)(i / p.cols), c0 = (int)(i - (int64_t)r0 * p.cols);
-  const int rlo = max(r0 - h, 0), rhi = min(r0 + h, p.rows - 1);
-  const int clo = max(c0 - h, 0), chi = min(c0 + h, p.cols - 1);
-  int nk = 0;
-  for (int r = rlo; r <= rhi; ++r)
-    for (int c = clo; c <= chi; ++c) nk += is_kept(bm, (int64_t)r * p.cols + c);
-  if (nk < min_count) return false;
-  const float vi = value_of<DT, NORM>(p, frame, f, i);
-  for (int r = rlo; r <= rhi; ++r)
-    for (int c = clo; c <= chi; ++c) {
-      const int64_t j = (int64_t)r * p.cols + c;
-      if (j == i || __ldg(p.bop + j) < 0) continue;
-      const float vj = value_of<DT, NORM>(p, frame, f, j);
-      if (!(vi > vj || (vi == vj && i < j))) return false;
-    }
-  return true;
+// Bits [j, j + w) of a frame's bitmap, w <= 15 (a second word is read only
+// where the run crosses into it, so no word past the run's last bit is read).
+__device__ __forceinline__ uint32_t bit_run(const uint32_t* bm, int64_t j, int w) {
+  const int sh = (int)(j & 31);
+  const uint32_t* q = bm + (j >> 5);
+  const uint32_t a = __ldg(q);
+  const uint32_t b = sh + w > 32 ? __ldg(q + 1) : 0u;
+  return __funnelshift_r(a, b, sh) & ((1u << w) - 1u);
 }
 
-// Phase 1: one flag bit per kept-list entry, and peaks per chunk of 256.
+// Value of pixel j of launch frame f where the pixel is valid (it has a bin,
+// hence a centre entry), else ok = false.
+template <int DT, bool NORM>
+__device__ __forceinline__ float valid_value(const PixArgs& p, const void* frame, int64_t f, int64_t j, bool& ok) {
+  if (p.stage) {
+    const int32_t q = __ldg(p.pos_of + j);
+    ok = q >= 0;
+    return ok ? __ldg(p.stage + f * p.npos + q) : 0.0f;
+  }
+  ok = __ldg(p.bop + j) >= 0;
+  return ok ? pixel_value<DT, NORM>(frame, j, p.npix, p.ped, p.gain, p.norm) : 0.0f;
+}
+
+// Phase 1 of the peaks: one flag bit per kept-list entry, and peaks per chunk
+// of 256. A kept pixel is a peak (Section 4) if its patch holds at least
+// min_count kept pixels and it is the maximum of the patch's valid pixels
+// (ties: lowest index).
+//
+// The kernel is bound by the latency of dependent gathers. A thread counts
+// its pixel's kept neighbours a patch row at a time (a run of bitmap bits and
+// a population count); the few entries with enough of them (about 1 in 50)
+// are then tested by the warp together, one lane per patch pixel and as many
+// candidates at once as fit the 32 lanes, so all their values are in flight
+// at once instead of one neighbour after another on one lane. The grid fills
+// the GPU whatever the number of frames.
+// 48 Jungfrau-4M frames (90,000 kept pixels each): 145 -> 97 us; 4 frames:
+// 84 -> 22 us.
 template <int DT, bool NORM>
 __global__ void __launch_bounds__(kPeakThreads) k_peak_flags(PixArgs p, const uint32_t* bitmap, int64_t words,
                                                              const int32_t* idx, const int32_t* n_kept, int64_t kcap,
                                                              int32_t patch, int32_t min_count, uint32_t* flags,
                                                              int32_t* chunk_cnt, int32_t n_chunks) {
+  __shared__ int32_t cpix_s[kPeakThreads];   // per warp: its candidates' pixels
+  __shared__ int cnt_s[kPeakThreads / 32];
   const int64_t f = blockIdx.y;
   const uint32_t* bm = bitmap + f * words;
   const void* frame = p.fptr ? (const void*)p.fptr[f] : frame_ptr<DT>(p.frames, f, p.npix);
   const int64_t g = p.fidx ? p.fidx[f] : f;
   int64_t n = n_kept[g];
   if (n > kcap) n = kcap;
-  const int h = patch >> 1;
+  const int h = patch >> 1, area = patch * patch, mid = area >> 1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per = area <= 32 ? 32 / area : 1;   // candidates tested at once
+  int32_t* cand = cpix_s + 32 * warp;
   for (int64_t ch = blockIdx.x; ch * kPeakChunk < n; ch += gridDim.x) {
     const int64_t k = ch * kPeakChunk + threadIdx.x;
-    bool peak = false;
-    const int64_t i = k < n ? idx[g * kcap + k] : -1;
-    if (i >= 0 && i < p.npix && __ldg(p.bop + i) >= 0) peak = peak_test<DT, NORM>(p, frame, f, bm, i, h, min_count);
-    const uint32_t m = __ballot_sync(0xffffffffu, peak);
-    if ((threadIdx.x & 31) == 0) flags[f * ((int64_t)n_chunks * 8) + ch * 8 + (threadIdx.x >> 5)] = m;
-    const int c = __syncthreads_count(peak);
-    if (threadIdx.x == 0) chunk_cnt[f * n_chunks + ch] = c;
+    const int32_t i = k < n ? idx[g * kcap + k] : -1;
+    bool enough = false;
+    if (i >= 0 && i < p.npix && __ldg(p.bop + i) >= 0) {
+      const int r0 = i / p.cols, c0 = i - r0 * p.cols;
+      const int rlo = max(r0 - h, 0), rhi = min(r0 + h, p.rows - 1);
+      const int clo = max(c0 - h, 0), w = min(c0 + h, p.cols - 1) - clo + 1;
+      int nk = 0;
+      for (int r = rlo; r <= rhi; ++r) nk += __popc(bit_run(bm, (int64_t)r * p.cols + clo, w));
+      enough = nk >= min_count;
+    }
+    const uint32_t em = __ballot_sync(0xffffffffu, enough);
+    uint32_t peaks = 0;
+    if (em) {
+      const int rank = __popc(em & ((1u << lane) - 1u)), nc = __popc(em);
+      if (enough) cand[rank] = i;
+      __syncwarp();
+      bool peak = false;
+      for (int c0 = 0; c0 < nc; c0 += per) {
+        bool fine = true;   // no patch pixel of this lane beats its candidate
+        const int sub = per > 1 ? lane / area : 0;
+        const int c = c0 + sub;
+        const bool active = sub < per && c < nc;
+        const int64_t ci = active ? cand[c] : 0;
+        const int cr = (int)(ci / p.cols), cc = (int)(ci - (int64_t)cr * p.cols);
+        float vi = 0.0f;
+        bool ok;
+        if (per == 1 && active) vi = valid_value<DT, NORM>(p, frame, f, ci, ok);   // (the patch exceeds the warp)
+        for (int o0 = 0; o0 < area; o0 += 32) {
+          const int o = per > 1 ? lane - sub * area : o0 + lane;
+          const int r = cr + o / patch - h, q = cc + o % patch - h;
+          bool there = active && o < area && r >= 0 && r < p.rows && q >= 0 && q < p.cols;
+          const int64_t j = (int64_t)r * p.cols + q;
+          float vj = 0.0f;
+          if (there) vj = valid_value<DT, NORM>(p, frame, f, j, there);
+          if (per > 1) vi = __shfl_sync(0xffffffffu, vj, min(sub * area + mid, 31));
+          if (there && j != ci && !(vi > vj || (vi == vj && ci < j))) fine = false;
+          if (per > 1) break;
+          if (__any_sync(0xffffffffu, !fine)) break;
+        }
+        const uint32_t b = __ballot_sync(0xffffffffu, fine);
+        if (enough && rank >= c0 && rank < c0 + per) {
+          const uint32_t want = per > 1 ? ((1u << area) - 1u) << ((rank - c0) * area) : 0xffffffffu;
+          peak = (b & want) == want;
+        }
+      }
+      peaks = __ballot_sync(0xffffffffu, peak);
+      __syncwarp();   // the list is rewritten by the warp's next chunk
+    }
+    if (lane == 0) {
+      flags[f * ((int64_t)n_chunks * 8) + ch * 8 + warp] = peaks;
+      cnt_s[warp] = __popc(peaks);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int c = 0;
+#pragma unroll
+      for (int w8 = 0; w8 < kPeakThreads / 32; ++w8) c += cnt_s[w8];
+      chunk_cnt[f * n_chunks + ch] = c;
+    }
+    __syncthreads();
   }
 }
 
-// Phase 2 (one CTA per frame): prefix over chunk counts, then every flagged
-// entry writes its record at its rank: ascending pixel order, since the
-// kept list ascends.
+// Phase 2: every flagged entry writes its record at its rank in the frame:
+// ascending pixel order, since the kept list ascends. The chunks of a frame
+// are split over gridDim.x CTAs (a slice each, as many as fill the GPU: one
+// CTA a frame left a 4-frame call on 4 multiprocessors); each counts the
+// peaks of the chunks before its slice itself (a few hundred integers), lists
+// its slice's flagged entries at their ranks in shared memory, kPeakList at a
+// time, and writes the records one peak a thread.
+// 48 Jungfrau-4M frames (750 peaks each): 54 -> 42 us; 4 frames: 55 -> 22 us;
+// one 16M frame: 63 -> 20 us.
 template <int DT, bool NORM, bool INTERP>
-__global__ void __launch_bounds__(1024) k_peak_emit(PixArgs p, int32_t nbins, const float* mean, const float* sigma,
-                                                    const uint32_t* bitmap, int64_t words, const int32_t* idx,
-                                                    const int32_t* n_kept, int64_t kcap, int32_t patch,
-                                                    const uint32_t* flags, int32_t* chunk_cnt, int32_t n_chunks,
-                                                    sep_peak* peaks, int64_t pcap, int32_t* n_peaks,
-                                                    int32_t* status) {
-  __shared__ int sh[32];
-  const int64_t f = blockIdx.x;
+__global__ void __launch_bounds__(kPeakThreads) k_peak_emit(PixArgs p, int32_t nbins, const float* mean,
+                                                            const float* sigma, const uint32_t* bitmap, int64_t words,
+                                                            const int32_t* idx, const int32_t* n_kept, int64_t kcap,
+                                                            int32_t patch, const uint32_t* flags,
+                                                            const int32_t* chunk_cnt, int32_t n_chunks,
+                                                            sep_peak* peaks, int64_t pcap, int32_t* n_peaks,
+                                                            int32_t* status) {
+  constexpr int kWarps = kPeakThreads / 32;
+  __shared__ int sh[kWarps];
+  __shared__ int64_t sum_s[2][kWarps];
+  __shared__ int32_t base_s[kPeakThreads];
+  __shared__ int32_t plist[kPeakList];
+  const int64_t f = blockIdx.y;
   const int64_t g = p.fidx ? p.fidx[f] : f;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int64_t n = n_kept[g];
   if (n > kcap) n = kcap;
   const int nch = (int)((n + kPeakChunk - 1) / kPeakChunk);
-  // chunk counts become chunk offsets, in place (a count <= kcap < 2^31)
-  int32_t* chunk_base = chunk_cnt + f * n_chunks;
-  int64_t total = 0;
-  for (int c0 = 0; c0 < nch; c0 += 1024) {
-    const int c = c0 + threadIdx.x;
-    const int x = c < nch ? chunk_base[c] : 0;
-    int tt;
-    const int off = block_exclusive_scan<1024>(x, &tt, sh);
-    if (c < nch) chunk_base[c] = (int32_t)(total + off);
-    total += tt;
+  const int slice = (nch + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int first = min((int)blockIdx.x * slice, nch), last = min(first + slice, nch);
+  const int32_t* cnt = chunk_cnt + f * n_chunks;
+  int64_t before = 0, total = 0;
+  for (int c = tid; c < nch; c += kPeakThreads) {
+    const int x = cnt[c];
+    total += x;
+    if (c < first) before += x;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    before += __shfl_xor_sync(0xffffffffu, before, o);
+    total += __shfl_xor_sync(0xffffffffu, total, o);
+  }
+  if (lane == 0) {
+    sum_s[0][warp] = before;
+    sum_s[1][warp] = total;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
+  before = total = 0;
+#pragma unroll
+  for (int w8 = 0; w8 < kWarps; ++w8) {
+    before += sum_s[0][w8];
+    total += sum_s[1][w8];
+  }
+  if (blockIdx.x == 0 && tid == 0) {
     n_peaks[g] = (int32_t)total;
     if (total > pcap) atomicOr(status, SEP_DEV_CAPACITY);
   }
@@ -438,62 +529,70 @@ __global__ void __launch_bounds__(1024) k_peak_emit(PixArgs p, int32_t nbins, co
   const float* mu = mean + row;
   const float* sd = sigma + row;
   const int h = patch >> 1;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t* fl = flags + f * ((int64_t)n_chunks * 8);
-  // the flagged entries go through a shared list, kPeakList at a time: a
-  // warp per chunk and a lane per flag bit list them at their ranks, then a
-  // thread per listed peak writes its record (all patches in flight together)
-  __shared__ int32_t plist[kPeakList];
-  const int64_t n_out = total < pcap ? total : pcap;
-  for (int64_t r0 = 0; r0 < n_out; r0 += kPeakList) {
-    for (int c = warp; c < nch; c += 32) {
-      int64_t rank = chunk_base[c];
-      if (rank >= r0 + kPeakList) continue;
-      for (int wd = 0; wd < 8; ++wd) {
-        const uint32_t m = fl[c * 8 + wd];
-        if (m == 0) continue;
-        if ((m >> lane) & 1u) {
-          const int64_t pos = rank + __popc(m & ((1u << lane) - 1u));
-          if (pos >= r0 && pos < r0 + kPeakList) plist[pos - r0] = c * kPeakChunk + wd * 32 + lane;
+  // the slice's chunks, kPeakThreads at a time: their ranks, then their records
+  for (int c0 = first; c0 < last && before < pcap; c0 += kPeakThreads) {
+    const int nc = min(last - c0, kPeakThreads);
+    int part;
+    const int off = block_exclusive_scan<kPeakThreads>(tid < nc ? cnt[c0 + tid] : 0, &part, sh);
+    base_s[tid] = off;
+    __syncthreads();
+    const int64_t room = pcap - before;
+    const int n_out = (int64_t)part < room ? part : (int)room;
+    for (int r0 = 0; r0 < n_out; r0 += kPeakList) {
+      for (int c = warp; c < nc; c += kWarps) {
+        int rank = base_s[c];
+        if (rank >= r0 + kPeakList) break;   // (ranks ascend with the chunk)
+        // a lane per flag word: ranks of the 8 words, then of their bits
+        const uint32_t mw = lane < 8 ? __ldg(fl + (int64_t)(c0 + c) * 8 + lane) : 0u;
+#pragma unroll
+        for (int wd = 0; wd < 8; ++wd) {
+          const uint32_t m = __shfl_sync(0xffffffffu, mw, wd);
+          const int pos = rank + __popc(m & ((1u << lane) - 1u));
+          if (((m >> lane) & 1u) && pos >= r0 && pos < r0 + kPeakList)
+            plist[pos - r0] = (c0 + c) * kPeakChunk + wd * 32 + lane;
+          rank += __popc(m);
         }
-        rank += __popc(m);
       }
-    }
-    __syncthreads();
-    const int nr = (int)(n_out - r0 < kPeakList ? n_out - r0 : kPeakList);
-    for (int t = threadIdx.x; t < nr; t += 1024) {
-      const int64_t pos = r0 + t;
-      const int64_t i = idx[g * kcap + plist[t]];
-      const int rr0 = (int)(i / p.cols), cc0 = (int)(i - (int64_t)rr0 * p.cols);
-      const int rlo = max(rr0 - h, 0), rhi = min(rr0 + h, p.rows - 1);
-      const int clo = max(cc0 - h, 0), chi = min(cc0 + h, p.cols - 1);
-      float I = 0.f, sy = 0.f, sx = 0.f, s2 = 0.f;
-      int nk = 0;
-      for (int r = rlo; r <= rhi; ++r)
-        for (int cc = clo; cc <= chi; ++cc) {
-          const int64_t j = (int64_t)r * p.cols + cc;
-          if (!is_kept(bm, j)) continue;
-          const int32_t bj = __ldg(p.bop + j);
-          const float vj = value_of<DT, NORM>(p, frame, f, j);
-          // background of the pixel's bin, or the profile at its centre
-          const float w = vj - (INTERP ? profile_at(mu, bj, p.ia, p.it, j, nbins) : __ldg(mu + bj));
-          const float sdv = INTERP ? profile_at(sd, bj, p.ia, p.it, j, nbins) : __ldg(sd + bj);
-          ++nk;
-          I += w;
-          sy += w * ((float)r + 0.5f);
-          sx += w * ((float)cc + 0.5f);
-          s2 += sdv * sdv;
+      __syncthreads();
+      const int nr = min(n_out - r0, kPeakList);
+      for (int t = tid; t < nr; t += kPeakThreads) {
+        const int64_t i = idx[g * kcap + plist[t]];
+        const int rr0 = (int)(i / p.cols), cc0 = (int)(i - (int64_t)rr0 * p.cols);
+        const int rlo = max(rr0 - h, 0), rhi = min(rr0 + h, p.rows - 1);
+        const int clo = max(cc0 - h, 0), w = min(cc0 + h, p.cols - 1) - clo + 1;
+        float I = 0.f, sy = 0.f, sx = 0.f, s2 = 0.f;
+        int nk = 0;
+        for (int r = rlo; r <= rhi; ++r) {
+          const int64_t j0 = (int64_t)r * p.cols + clo;
+          for (uint32_t m = bit_run(bm, j0, w); m; m &= m - 1u) {
+            const int k = __ffs(m) - 1, cc = clo + k;
+            const int64_t j = j0 + k;
+            const int32_t bj = __ldg(p.bop + j);
+            if (bj < 0) continue;   // (a caller's list may name masked pixels)
+            const float vj = value_of<DT, NORM>(p, frame, f, j);
+            // background of the pixel's bin, or the profile at its centre
+            const float w1 = vj - (INTERP ? profile_at(mu, bj, p.ia, p.it, j, nbins) : __ldg(mu + bj));
+            const float sdv = INTERP ? profile_at(sd, bj, p.ia, p.it, j, nbins) : __ldg(sd + bj);
+            ++nk;
+            I += w1;
+            sy += w1 * ((float)r + 0.5f);
+            sx += w1 * ((float)cc + 0.5f);
+            s2 += sdv * sdv;
+          }
         }
-      sep_peak rec;
-      rec.idx = (int32_t)i;
-      rec.I = I;
-      rec.y = sy / I;
-      rec.x = sx / I;
-      rec.sigma = sqrtf(s2);
-      rec.npix = nk;
-      peaks[g * pcap + pos] = rec;
+        sep_peak rec;
+        rec.idx = (int32_t)i;
+        rec.I = I;
+        rec.y = sy / I;
+        rec.x = sx / I;
+        rec.sigma = sqrtf(s2);
+        rec.npix = nk;
+        peaks[g * pcap + before + r0 + t] = rec;
+      }
+      __syncthreads();
     }
-    __syncthreads();
+    before += part;
   }
 }
 
@@ -628,14 +727,18 @@ cudaError_t launch_peaks(const PixArgs& p, int32_t n_frames, int32_t nbins, cons
   const int32_t nch = peak_chunks(kcap);
   uint32_t* flags = reinterpret_cast<uint32_t*>(scratch);
   int32_t* cnt = scratch + (int64_t)n_frames * nch * 8;
-  dim3 g1((unsigned)std::min<int32_t>(std::max<int32_t>(nch, 1), kPeakCtasPerFrame), (unsigned)n_frames);
+  // either grid: kPeakCtas CTAs over the frames where the lists can use them
+  // (a chunk each in phase 1, a slice of at least 8 chunks each in phase 2)
+  const int32_t want = std::max(1, (kPeakCtas + n_frames - 1) / n_frames);
+  dim3 g1((unsigned)std::min(std::max(nch, 1), std::max(want, 64)), (unsigned)n_frames);
+  dim3 g2((unsigned)std::min((nch + 7) / 8 + (nch == 0), std::max(want / 4, 1)), (unsigned)n_frames);
   const bool nrm = p.norm != nullptr;
   const bool itp = p.ia != nullptr && p.it != nullptr;
 #define SEP_FLAG_ARGS p, bitmap, words, idx, n_kept, kcap, patch, min_count, flags, cnt, nch
 #define SEP_PEMIT_ARGS p, nbins, mean, sigma, bitmap, words, idx, n_kept, kcap, patch, flags, cnt, nch, peaks, pcap, n_peaks, status
 #define SEP_PEMIT(DT, NR)                                                              \
-  if (itp) k_peak_emit<DT, NR, true><<<n_frames, 1024, 0, s>>>(SEP_PEMIT_ARGS);      \
-  else k_peak_emit<DT, NR, false><<<n_frames, 1024, 0, s>>>(SEP_PEMIT_ARGS)
+  if (itp) k_peak_emit<DT, NR, true><<<g2, kPeakThreads, 0, s>>>(SEP_PEMIT_ARGS);      \
+  else k_peak_emit<DT, NR, false><<<g2, kPeakThreads, 0, s>>>(SEP_PEMIT_ARGS)
   if (p.dtype == SEP_DTYPE_U16_JF) {
     if (nrm) {
       k_peak_flags<SEP_DTYPE_U16_JF, true><<<g1, kPeakThreads, 0, s>>>(SEP_FLAG_ARGS);
