@@ -56,21 +56,172 @@ __global__ void k_thresholds(const float* mean, const float* sigma, float k_pick
 }
 
 // One thread per pixel, one warp per bitmap word: every word is written.
+// Level of pixel i in a per-bin profile p (bin level, or the radial
+// interpolation between the bins a and a + 1 with weight t on the upper).
+__device__ __forceinline__ float profile_at(const float* p, int32_t b, const int32_t* ia, const float* it, int64_t i,
+                                            int32_t nbins) {
+  if (!ia) return __ldg(p + b);
+  const int32_t a = __ldg(ia + i);
+  const float t = __ldg(it + i);
+  const float hi = a + 1 < nbins ? __ldg(p + a + 1) : 0.0f;
+  return __fadd_rn(__fmul_rn(__fsub_rn(1.0f, t), __ldg(p + a)), __fmul_rn(t, hi));
+}
+
+// Pixels that a thread of the image-order kernels takes from each frame, 32
+// apart: a warp covers 128 consecutive pixels, every access of it is
+// coalesced whatever the alignment of the frame, and a ballot is a word of
+// the bitmap.
+constexpr int kPixPerThread = 4;
+constexpr int kImageThreads = 256;
+constexpr int kPixPerCta = kImageThreads * kPixPerThread;
+
+// Frames a thread of the image-order kernels walks: the pixels' tables
+// (calibration, bins) are read once for all of them, as long as the grid
+// still holds four waves of 8 CTAs on every multiprocessor; the groups of a
+// batch are even.
+int32_t frames_per_thread(int32_t n_frames, int64_t ctas) {
+  const int32_t most = (int32_t)std::min<int64_t>(std::max<int64_t>(ctas * n_frames / (152 * 8 * 4), 1), 16);
+  const int32_t groups = (n_frames + most - 1) / most;
+  return (n_frames + groups - 1) / groups;
+}
+
+// Four pixels of a warp's 128 (32 apart from i0), for the frames a thread
+// walks: their tables, and their values frame by frame. Pixels past the last
+// read the last one's words, and pixels without a bin take no part in the
+// tests of value(): neither costs the loop over the frames a branch.
 template <int DT, bool NORM>
-__global__ void k_mark(PixArgs p, int32_t nbins, const float* thr, uint32_t* bitmap, int64_t words) {
-  const int64_t f = blockIdx.y;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  bool keep = false;
-  if (i < p.npix) {
-    int32_t b = __ldg(p.bop + i);
-    if (b >= 0) {
-      float v = pixel_value<DT, NORM>(frame_ptr<DT>(p.frames, f, p.npix), i, p.npix, p.ped, p.gain, p.norm);
-      keep = v > __ldg(thr + f * nbins + b);
+struct PixelColumn {
+  Level0 cal[kPixPerThread];
+  float nm[kPixPerThread];
+  uint32_t w[kPixPerThread];   // the words of the frame loaded last
+  uint32_t i[kPixPerThread];   // the pixels, at most npix - 1 (32-bit offsets: one instruction an address)
+  bool valid[kPixPerThread];   // inside the image, and with a bin
+  __device__ __forceinline__ PixelColumn(const PixArgs& p, int64_t i0) {
+#pragma unroll
+    for (int k = 0; k < kPixPerThread; ++k) {
+      i[k] = (uint32_t)min(i0 + 32 * k, p.npix - 1);
+      valid[k] = i0 + 32 * k < p.npix && __ldg(p.bop + i[k]) >= 0;
+      nm[k] = 1.0f;
+      if (DT == SEP_DTYPE_U16_JF) {
+        cal[k].set(__ldg(p.ped + i[k]), __ldg(p.gain + i[k]));
+        if (!valid[k]) cal[k].limit = 0xffffffffu;
+      }
+      if (NORM) nm[k] = __ldg(p.norm + i[k]);
     }
   }
-  uint32_t m = __ballot_sync(0xffffffffu, keep);
-  if ((threadIdx.x & 31) == 0 && (i >> 5) < words) bitmap[f * words + (i >> 5)] = m;
+  __device__ __forceinline__ const void* frame(const PixArgs& p, int64_t f) const {
+    return p.fptr ? (const void*)p.fptr[f] : frame_ptr<DT>(p.frames, f, p.npix);
+  }
+  __device__ __forceinline__ void load(const PixArgs& p, int64_t f) {
+    const void* fr = frame(p, f);
+#pragma unroll
+    for (int k = 0; k < kPixPerThread; ++k) {
+      if (DT == SEP_DTYPE_U16_JF) w[k] = __ldg(reinterpret_cast<const uint16_t*>(fr) + i[k]);
+      else w[k] = __float_as_uint(__ldg(reinterpret_cast<const float*>(fr) + i[k]));
+    }
+  }
+  // the values of frame f's words u: pixel_value(), bit for bit, for the
+  // valid pixels
+  __device__ __forceinline__ void values(const PixArgs& p, int64_t f, const uint32_t (&u)[kPixPerThread],
+                                         float (&x)[kPixPerThread]) const {
+    bool rest = false;
+#pragma unroll
+    for (int k = 0; k < kPixPerThread; ++k) {
+      x[k] = DT == SEP_DTYPE_U16_JF ? cal[k].value(u[k]) : __uint_as_float(u[k]);
+      if (DT == SEP_DTYPE_U16_JF) rest = rest || u[k] >= cal[k].limit;
+      if (NORM) x[k] = __fdiv_rn(x[k], nm[k]);
+    }
+    if (DT != SEP_DTYPE_U16_JF || !rest) return;
+    // another gain level or an unusual calibration
+#pragma unroll
+    for (int k = 0; k < kPixPerThread; ++k)
+      if (u[k] >= cal[k].limit)
+        x[k] = pixel_value<DT, NORM>(frame(p, f), i[k], p.npix, p.ped, p.gain, p.norm);
+  }
+};
+
+// v > RD32(m + k s) with the sum in binary64: for a binary32 v that is
+// v > RN64(m + k s). Decided in binary32 when v is further from the sum than
+// binary32 can be off it (t is within 2^-24 of the sum, the difference within
+// 2^-24 of itself), else, and for NaN and infinities, in binary64, whose
+// rate on this GPU is a small fraction of binary32's (out of line, or the
+// compiler computes both sides of the choice: 242 us instead of 70 for the
+// float frames named below).
+static __device__ __noinline__ bool above_threshold64(float v, float m, float s, float k) {
+  return v > __double2float_rd((double)m + (double)k * (double)s);
 }
+__device__ __forceinline__ bool above_threshold(float v, float m, float s, float k) {
+  const float t = __fmaf_rn(k, s, m);
+  const float d = __fsub_rn(v, t);
+  bool above = d > 0.0f;
+  if (!(fabsf(d) > __fmaf_rn(0x1p-21f, fabsf(t), 0x1p-120f))) above = above_threshold64(v, m, s, k);
+  return above;
+}
+
+// Kept-pixel bitmap of a batch in image order (Section 3). The threshold of a
+// pixel is its bin's (thr [F][nbins]), or, INTERP, RD(mu(x) + k_pick sigma(x))
+// from the frame's profile interpolated at the pixel centre. Values are
+// corrected from the frame's words: in image order those are one contiguous
+// stream, where the staged copy of a batch would cost a sector a pixel. A
+// warp writes four words of the bitmap at once, every word of the row
+// (pixels past the last count as dropped).
+//
+// One pixel a thread and frame was bound by its instructions: an IEEE
+// division with its tables, a bin, and with INTERP a binary64 sum a pixel
+// (16 raw Jungfrau-4M frames: 314 -> 99 us; INTERP, 29 float frames of 1.1
+// Mpixel: 301 -> 70 us). It still is: 73 % of the issue slots are taken. The
+// register bound keeps 40 warps on a multiprocessor (76 registers without
+// it, 149 us).
+template <int DT, bool NORM, bool INTERP>
+__global__ void __launch_bounds__(kImageThreads, 5) k_mark(PixArgs p, int32_t n_frames, int32_t frames_per_cta,
+                                                        int32_t nbins, const float* thr, const float* mean,
+                                                        const float* sigma, float k_pick, uint32_t* bitmap,
+                                                        int64_t words) {
+  const int lane = threadIdx.x & 31;
+  const int64_t w0 = ((int64_t)blockIdx.x * (kImageThreads / 32) + (threadIdx.x >> 5)) * kPixPerThread;
+  if (w0 >= words) return;   // (words is a multiple of 8)
+  PixelColumn<DT, NORM> px(p, w0 * 32 + lane);
+  uint32_t b[kPixPerThread];   // the bin (INTERP: the lower bin)
+  float t[kPixPerThread];
+  uint32_t valid[kPixPerThread];
+#pragma unroll
+  for (int k = 0; k < kPixPerThread; ++k) {
+    valid[k] = __ballot_sync(0xffffffffu, px.valid[k]);
+    t[k] = INTERP ? __ldg(p.it + px.i[k]) : 0.0f;
+    b[k] = (uint32_t)(INTERP ? __ldg(p.ia + px.i[k]) : max(__ldg(p.bop + px.i[k]), 0));
+  }
+  const int32_t f0 = blockIdx.y * frames_per_cta, f1 = min(f0 + frames_per_cta, n_frames);
+  px.load(p, f0);
+  for (int32_t f = f0; f < f1; ++f) {
+    uint32_t w[kPixPerThread];
+#pragma unroll
+    for (int k = 0; k < kPixPerThread; ++k) w[k] = px.w[k];
+    if (f + 1 < f1) px.load(p, f + 1);   // the next frame's words are under way meanwhile
+    const int64_t row = INTERP && p.orow ? p.orow[f] : f * (int64_t)nbins;
+    const float* mu = INTERP ? mean + row : thr + row;   // the frame's profile, or its thresholds
+    const float* sd = INTERP ? sigma + row : nullptr;
+    float x[kPixPerThread];
+    px.values(p, f, w, x);
+    uint32_t m[kPixPerThread];
+#pragma unroll
+    for (int k = 0; k < kPixPerThread; ++k) {
+      bool keep;
+      if (INTERP) {
+        const bool up = (int32_t)b[k] + 1 < nbins;
+        const float m0 = __ldg(mu + b[k]), m1 = up ? __ldg(mu + b[k] + 1) : 0.0f;
+        const float s0 = __ldg(sd + b[k]), s1 = up ? __ldg(sd + b[k] + 1) : 0.0f;
+        const float u = __fsub_rn(1.0f, t[k]);
+        keep = above_threshold(x[k], __fadd_rn(__fmul_rn(u, m0), __fmul_rn(t[k], m1)),
+                               __fadd_rn(__fmul_rn(u, s0), __fmul_rn(t[k], s1)), k_pick);
+      } else {
+        keep = x[k] > __ldg(mu + b[k]);
+      }
+      m[k] = __ballot_sync(0xffffffffu, keep) & valid[k];
+    }
+    if (lane == 0) *reinterpret_cast<uint4*>(bitmap + f * words + w0) = make_uint4(m[0], m[1], m[2], m[3]);
+  }
+}
+static_assert(kPixPerThread == 4, "a warp writes its four words as one vector");
 
 // Staged values back to image order; pixels without a position get NaN.
 __global__ void k_unstage(const float* stage, int64_t stride, const int32_t* pos_of, int64_t npix, float* out) {
@@ -197,17 +348,6 @@ __global__ void __launch_bounds__(kCompactThreads) k_emit_kept(PixArgs p, const 
 // Densification (Section 3): the background level of every binned pixel
 // (its bin's mean, or RN(mean + RN(sigma z)) with the caller's deviates z),
 // fill where a pixel has no bin; one thread per pixel.
-// Level of pixel i in a per-bin profile p (bin level, or the radial
-// interpolation between the bins a and a + 1 with weight t on the upper).
-__device__ __forceinline__ float profile_at(const float* p, int32_t b, const int32_t* ia, const float* it, int64_t i,
-                                            int32_t nbins) {
-  if (!ia) return __ldg(p + b);
-  const int32_t a = __ldg(ia + i);
-  const float t = __ldg(it + i);
-  const float hi = a + 1 < nbins ? __ldg(p + a + 1) : 0.0f;
-  return __fadd_rn(__fmul_rn(__fsub_rn(1.0f, t), __ldg(p + a)), __fmul_rn(t, hi));
-}
-
 __global__ void __launch_bounds__(256) k_dense_background(const int32_t* bop, int64_t npix, int32_t nbins,
                                                           const float* mean, const float* sigma,
                                                           const float* noise, float fill, const int32_t* ia,
@@ -252,31 +392,6 @@ __global__ void __launch_bounds__(256) k_dense_background4(const int32_t* bop, i
     }
   }
   *reinterpret_cast<float4*>(out + f * npix + i) = make_float4(x[0], x[1], x[2], x[3]);
-}
-
-// Kept pixels against the smooth background (Section 3): the threshold of
-// pixel i is RD(mu(x_i) + k_pick sigma(x_i)) with the frame's profile
-// interpolated at the pixel centre. One thread per pixel, one warp per
-// bitmap word: every word is written.
-template <int DT, bool NORM>
-__global__ void __launch_bounds__(256) k_mark_interp(PixArgs p, int32_t nbins, const float* mean, const float* sigma,
-                                                     float k_pick, uint32_t* bitmap, int64_t words) {
-  const int64_t f = blockIdx.y;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  bool keep = false;
-  if (i < p.npix) {
-    const int32_t b = __ldg(p.bop + i);
-    if (b >= 0) {
-      const int64_t row = p.orow ? p.orow[f] : f * (int64_t)nbins;
-      const float m = profile_at(mean + row, b, p.ia, p.it, i, nbins);
-      const float sd = profile_at(sigma + row, b, p.ia, p.it, i, nbins);
-      const void* frame = p.fptr ? (const void*)p.fptr[f] : frame_ptr<DT>(p.frames, f, p.npix);
-      const float v = value_of<DT, NORM>(p, frame, f, i);
-      keep = v > __double2float_rd((double)m + (double)k_pick * (double)sd);
-    }
-  }
-  const uint32_t mk = __ballot_sync(0xffffffffu, keep);
-  if ((threadIdx.x & 31) == 0 && (i >> 5) < words) bitmap[f * words + (i >> 5)] = mk;
 }
 
 // ... then the recorded values of the kept pixels.
@@ -613,36 +728,35 @@ cudaError_t launch_unstage(const float* stage, int64_t stride, const int32_t* po
   return cudaGetLastError();
 }
 
+namespace {
+template <bool INTERP>
+cudaError_t launch_mark_t(const PixArgs& p, int32_t n_frames, int32_t nbins, const float* thr, const float* mean,
+                          const float* sigma, float k_pick, uint32_t* bitmap, int64_t words, cudaStream_t s) {
+  if (n_frames <= 0) return cudaSuccess;
+  const int64_t ctas = (words * 32 + kPixPerCta - 1) / kPixPerCta;
+  const int32_t fpc = frames_per_thread(n_frames, ctas);
+  dim3 grid((unsigned)ctas, (unsigned)((n_frames + fpc - 1) / fpc));
+#define SEP_MARK_ARGS p, n_frames, fpc, nbins, thr, mean, sigma, k_pick, bitmap, words
+  if (p.dtype == SEP_DTYPE_U16_JF) {
+    if (p.norm) k_mark<SEP_DTYPE_U16_JF, true, INTERP><<<grid, kImageThreads, 0, s>>>(SEP_MARK_ARGS);
+    else k_mark<SEP_DTYPE_U16_JF, false, INTERP><<<grid, kImageThreads, 0, s>>>(SEP_MARK_ARGS);
+  } else {
+    if (p.norm) k_mark<SEP_DTYPE_F32, true, INTERP><<<grid, kImageThreads, 0, s>>>(SEP_MARK_ARGS);
+    else k_mark<SEP_DTYPE_F32, false, INTERP><<<grid, kImageThreads, 0, s>>>(SEP_MARK_ARGS);
+  }
+#undef SEP_MARK_ARGS
+  return cudaGetLastError();
+}
+}  // namespace
+
 cudaError_t launch_mark(const PixArgs& p, int32_t n_frames, int32_t nbins, const float* thr, uint32_t* bitmap,
                         int64_t words, cudaStream_t s) {
-  if (n_frames <= 0) return cudaSuccess;
-  dim3 grid((unsigned)((words * 32 + 255) / 256), (unsigned)n_frames);
-  const bool nrm = p.norm != nullptr;
-  if (p.dtype == SEP_DTYPE_U16_JF) {
-    if (nrm) k_mark<SEP_DTYPE_U16_JF, true><<<grid, 256, 0, s>>>(p, nbins, thr, bitmap, words);
-    else k_mark<SEP_DTYPE_U16_JF, false><<<grid, 256, 0, s>>>(p, nbins, thr, bitmap, words);
-  } else {
-    if (nrm) k_mark<SEP_DTYPE_F32, true><<<grid, 256, 0, s>>>(p, nbins, thr, bitmap, words);
-    else k_mark<SEP_DTYPE_F32, false><<<grid, 256, 0, s>>>(p, nbins, thr, bitmap, words);
-  }
-  return cudaGetLastError();
+  return launch_mark_t<false>(p, n_frames, nbins, thr, nullptr, nullptr, 0.0f, bitmap, words, s);
 }
 
 cudaError_t launch_mark_interp(const PixArgs& p, int32_t n_frames, int32_t nbins, const float* mean,
                                const float* sigma, float k_pick, uint32_t* bitmap, int64_t words, cudaStream_t s) {
-  if (n_frames <= 0) return cudaSuccess;
-  dim3 grid((unsigned)((words * 32 + 255) / 256), (unsigned)n_frames);
-  const bool nrm = p.norm != nullptr;
-#define SEP_MARK_ARGS p, nbins, mean, sigma, k_pick, bitmap, words
-  if (p.dtype == SEP_DTYPE_U16_JF) {
-    if (nrm) k_mark_interp<SEP_DTYPE_U16_JF, true><<<grid, 256, 0, s>>>(SEP_MARK_ARGS);
-    else k_mark_interp<SEP_DTYPE_U16_JF, false><<<grid, 256, 0, s>>>(SEP_MARK_ARGS);
-  } else {
-    if (nrm) k_mark_interp<SEP_DTYPE_F32, true><<<grid, 256, 0, s>>>(SEP_MARK_ARGS);
-    else k_mark_interp<SEP_DTYPE_F32, false><<<grid, 256, 0, s>>>(SEP_MARK_ARGS);
-  }
-#undef SEP_MARK_ARGS
-  return cudaGetLastError();
+  return launch_mark_t<true>(p, n_frames, nbins, nullptr, mean, sigma, k_pick, bitmap, words, s);
 }
 
 int32_t compact_tiles(int64_t words) { return (int32_t)((words + kTileWords - 1) / kTileWords); }

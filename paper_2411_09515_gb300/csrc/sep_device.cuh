@@ -31,6 +31,37 @@ __device__ __forceinline__ float pixel_value(const void* frame, int64_t col, int
   return p;
 }
 
+// Level-0 calibration of one pixel, for threads that correct the same pixel
+// of many frames: the pedestal, the gain, r = RN(1 / gain), and the words
+// that value() takes, those below limit (2^14: level 0; 0 where gain or
+// pedestal lie outside the range its correction step is exact in). The other
+// words go through pixel_value().
+//
+// RN((adc - ped) / gain) needs no division: with d = RN(adc - ped) and
+// q = RN(d r), the residual e = d - q gain is exact under a fused
+// multiply-add, and RN(q + e r) is the correctly rounded quotient
+// (Markstein's correction, IBM J. Res. Dev. 34(1), 1990) as long as gain,
+// quotient and residual are normal: with the ranges below a d other than 0
+// lies between 2^-83 and 2^61 (the spacing of the larger of adc and ped
+// bounds it below) and q between 2^-124 and 2^102; d = 0 gives the
+// quotient's zero.
+struct Level0 {
+  float ped = 0.0f, gain = 1.0f, r = 1.0f;
+  uint32_t limit = 0;
+  __device__ __forceinline__ void set(float p, float g) {
+    ped = p;
+    gain = g;
+    r = __frcp_rn(g);
+    const float ag = fabsf(g), ap = fabsf(p);
+    limit = ag >= 0x1p-40f && ag <= 0x1p40f && (p == 0.0f || (ap >= 0x1p-60f && ap <= 0x1p60f)) ? 0x4000u : 0u;
+  }
+  __device__ __forceinline__ float value(uint32_t u) const {
+    const float d = __fsub_rn((float)u, ped);
+    const float q = __fmul_rn(d, r);
+    return __fmaf_rn(__fmaf_rn(-q, gain, d), r, q);
+  }
+};
+
 template <int DT>
 __device__ __forceinline__ const void* frame_ptr(const void* frames, int64_t f, int64_t npix) {
   if (DT == SEP_DTYPE_U16_JF) return reinterpret_cast<const uint16_t*>(frames) + f * npix;
