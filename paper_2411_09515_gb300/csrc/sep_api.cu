@@ -669,11 +669,8 @@ sep_status sep_correct(sep_ctx* ctx, const sep_csr* csr, const sep_calib* calib,
   if (st != SEP_OK) return st;
   if (n_frames > 0 && !out_dev) return fail(ctx, SEP_ERR_ARG, "NULL output");
   if (n_frames == 0) return SEP_OK;
-  if ((st = ensure_stage(ctx, stage_stride(csr) * n_frames)) != SEP_OK) return st;
-  cudaStream_t s = (cudaStream_t)stream;
-  cudaError_t e = enqueue_stage(ctx, csr, calib, frames_dev, nullptr, dtype, n_frames, ctx->d_stage, s);
-  if (e == cudaSuccess)
-    e = sep::launch_unstage(ctx->d_stage, stage_stride(csr), csr->d_pos_of, csr->npix, n_frames, out_dev, s);
+  const cudaError_t e =
+      sep::launch_correct(pix_args(csr, calib, frames_dev, dtype), n_frames, out_dev, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "correct launch");
   return SEP_OK;
 }

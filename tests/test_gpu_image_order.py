@@ -1,4 +1,4 @@
-"""The image-order kernels (kept-pixel marks) against NumPy at the sizes where
+"""The image-order kernels (kept-pixel marks, corrected frames) against NumPy at the sizes where
 they can go wrong: fewer pixels than a warp's 128, one more, bitmap words that
 end inside a warp, frame counts that leave a remainder behind a thread's group
 of frames, frames at addresses aligned to one word only, and values on,
@@ -26,6 +26,19 @@ def _det(rows, cols, nbins):
 def _values(words, cal, norm):
     v = words if cal is None else np.stack([oracle.jf_photons(w, cal[0], cal[1]) for w in words])
     return v.astype(np.float32) if norm is None else (v.astype(np.float32) / norm).astype(np.float32)
+
+
+def _calib(n, rng):
+    """A Jungfrau calibration with pixels outside the usual range: gains near powers of two and near all-ones
+    significands, zero, tiny and huge pedestals and gains (the division-free path's limits and beyond them)."""
+    ped, gain = synth.jf_calib(n, seed=4)
+    at = rng.permutation(n)
+    for k, g in enumerate([1.0, np.nextafter(np.float32(2), np.float32(0)), 3.0, 2.0 ** -40, 2.0 ** 40, 2.0 ** -41,
+                           2.0 ** 41, 1e-38, 1e38, -7.0]):
+        gain[0, at[k::31]] = g
+    for k, p in enumerate([0.0, 2.0 ** -60, 2.0 ** 60, 1e-30, 1e30, 16383.0, 0.5]):
+        ped[0, at[k + 11::37]] = p
+    return ped, gain
 
 
 def _unaligned(a):
@@ -59,7 +72,7 @@ def test_sparsify_marks(rows, cols, F, raw, with_norm, smooth):
     det = _det(rows, cols, nbins=min(40, max(2, rows * cols // 20)))
     n = det.npix
     norm = rng.uniform(0.5, 2.0, n).astype(np.float32) if with_norm else None
-    cal = synth.jf_calib(n, seed=4) if raw else None
+    cal = _calib(n, rng) if raw else None
     mask = (rng.random(n) < 0.1).astype(np.uint8)
     sep = Separator.from_detector(det, mask=mask, norm=norm, calib=cal)
     sep.set_params(interpolate=smooth, k_pick=2.7)
@@ -99,4 +112,32 @@ def test_sparsify_marks(rows, cols, F, raw, with_norm, smooth):
         assert np.array_equal(idx[f, :want.size], want), f
         assert np.array_equal(val[f, :want.size].view(np.uint32), v[f, want].view(np.uint32)), f
     assert sep.device_status() == 0
+    sep.close()
+
+
+@pytest.mark.parametrize("raw,with_norm", [(False, False), (False, True), (True, False), (True, True)])
+@pytest.mark.parametrize("rows,cols,F", SIZES)
+def test_corrected_frames(rows, cols, F, raw, with_norm):
+    rng = np.random.default_rng(7 * rows * cols + F)
+    det = _det(rows, cols, nbins=min(40, max(2, rows * cols // 20)))
+    n = det.npix
+    norm = rng.uniform(0.5, 2.0, n).astype(np.float32) if with_norm else None
+    cal = _calib(n, rng) if raw else None
+    mask = (rng.random(n) < 0.1).astype(np.uint8)
+    sep = Separator.from_detector(det, mask=mask, norm=norm, calib=cal)
+    if raw:
+        words = rng.integers(0, 1 << 16, (F, n), dtype=np.uint16)
+    else:
+        words = rng.normal(3, 10, (F, n)).astype(np.float32)
+        words[:, ::17], words[:, 5::29] = np.nan, np.inf
+    with np.errstate(over="ignore", under="ignore"):
+        v = _values(words, cal, norm)
+    used = mask == 0
+    aligned = torch.from_numpy(words.view(np.int16) if raw else words).cuda()   # (vector accesses where they fit)
+    for frames in (_unaligned(words), aligned):
+        got = sep.correct(frames).cpu().numpy()
+        assert np.isnan(got[:, ~used]).all()
+        a, b = got[:, used], v[:, used]
+        assert np.array_equal(np.isnan(a), np.isnan(b))
+        assert np.array_equal(a[~np.isnan(a)].view(np.uint32), b[~np.isnan(b)].view(np.uint32))
     sep.close()
