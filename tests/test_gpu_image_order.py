@@ -1,4 +1,4 @@
-"""The image-order kernels (kept-pixel marks, corrected frames) against NumPy at the sizes where
+"""The image-order kernels (kept-pixel marks, corrected and dense frames) against NumPy at the sizes where
 they can go wrong: fewer pixels than a warp's 128, one more, bitmap words that
 end inside a warp, frame counts that leave a remainder behind a thread's group
 of frames, frames at addresses aligned to one word only, and values on,
@@ -140,4 +140,36 @@ def test_corrected_frames(rows, cols, F, raw, with_norm):
         a, b = got[:, used], v[:, used]
         assert np.array_equal(np.isnan(a), np.isnan(b))
         assert np.array_equal(a[~np.isnan(a)].view(np.uint32), b[~np.isnan(b)].view(np.uint32))
+    sep.close()
+
+
+@pytest.mark.parametrize("smooth", [False, True])
+@pytest.mark.parametrize("noisy", [False, True])
+@pytest.mark.parametrize("rows,cols,F", SIZES)
+def test_dense_background(rows, cols, F, noisy, smooth):
+    rng = np.random.default_rng(3 * rows * cols + F)
+    det = _det(rows, cols, nbins=min(40, max(2, rows * cols // 20)))
+    n = det.npix
+    mask = (rng.random(n) < 0.1).astype(np.uint8)
+    sep = Separator.from_detector(det, mask=mask)
+    bop = B.sep_csr_export(sep.csr)["bin_of_pixel"]
+    mean = rng.uniform(0.2, 30, (F, det.nbins)).astype(np.float32)
+    sigma = rng.uniform(0.1, 3, (F, det.nbins)).astype(np.float32)
+    z = rng.standard_normal((F, n)).astype(np.float32) if noisy else None
+
+    def at(p):
+        if not smooth:
+            return p[:, np.maximum(bop, 0)]
+        a, t = B.sep_csr_interp(sep.csr)
+        hi = np.where(a + 1 < p.shape[1], p[:, np.minimum(a + 1, p.shape[1] - 1)], np.float32(0))
+        return ((np.float32(1) - t) * p[:, a]).astype(np.float32) + (t * hi).astype(np.float32)
+
+    want = at(mean)
+    if noisy:
+        want = (want + (at(sigma) * z).astype(np.float32)).astype(np.float32)
+    want = np.where(bop >= 0, want, np.float32(-2.5)).astype(np.float32)
+    got = sep.densify(torch.from_numpy(mean).cuda(), torch.from_numpy(sigma).cuda(), None, None, None,
+                      noise=None if z is None else _unaligned(z), fill=-2.5, interpolate=smooth)
+    torch.cuda.synchronize()
+    assert np.array_equal(got.cpu().numpy().view(np.uint32), want.view(np.uint32))
     sep.close()
