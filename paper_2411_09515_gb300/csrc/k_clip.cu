@@ -107,8 +107,14 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 
 // Smallest float >= hi + lo and largest float <= hi + lo for a normalised
 // pair (hi = RN(hi + lo)).
-__device__ __forceinline__ float round_up_pair(float hi, float lo) { return lo > 0.0f ? nextafterf(hi, INFINITY) : hi; }
-__device__ __forceinline__ float round_dn_pair(float hi, float lo) { return lo < 0.0f ? nextafterf(hi, -INFINITY) : hi; }
+// (next binary32 value up or down from its bit pattern; lo is NaN or 0, so
+// hi stays, where hi is not finite)
+__device__ __forceinline__ float round_up_pair(float hi, float lo) {
+  const int b = __float_as_int(hi);
+  const int up = hi == 0.0f ? 1 : b + (b < 0 ? -1 : 1);
+  return lo > 0.0f ? __int_as_float(up) : hi;
+}
+__device__ __forceinline__ float round_dn_pair(float hi, float lo) { return -round_up_pair(-hi, -lo); }
 
 // Mean and deviation of one set from its shifted sums (each lane of the
 // item's warp, on the same totals):
@@ -338,15 +344,21 @@ __device__ __forceinline__ void unpack_totals(const float* th, const float* tl, 
 // or above C (no core entry can exceed it), else from a scan of the row.
 //
 // A warp owns its item from the first load to the marks. The row is read
-// straight from the staged frame (slot = entry, so a bin's values are one
-// contiguous run: 16-byte loads, several in flight per lane); only the tail
-// lives in shared memory, so many items fit an SM. Every total is a warp
+// from the staged frame (slot = entry, so a bin's values are one contiguous
+// run) through a small ring (stream_row); only that and the tail live in
+// shared memory, so many items fit an SM (15 for the longest rows of a
+// Jungfrau 4M). The kernel is bound by its instructions (9,700 a bin and frame
+// there: half of them the 5.5 replay steps, 40 % the scan of the row) at 61 %
+// of the issue slots, which its 15 warps do not fill further: 48 Jungfrau-4M
+// frames 925 -> 700 us, 4 frames 190 -> 150 us. Every total is a warp
 // butterfly, which leaves bit-identical totals on all lanes (addition, and
 // the error-free pair sum, are commutative), so every lane evaluates each
 // clip step itself: no lane waits for another, and the warps of a CTA
 // (other frames of the same bin) meet only between units of work.
 constexpr float kCoreMargin = 1.0f;   // core margin inside the clip interval, in deviations
 constexpr int kLoadsAhead = 4;        // 16-byte loads in flight per lane in a scan of the row
+constexpr int kRing = 4;              // groups under way per lane in a walk of the row
+constexpr int kMarkList = kRing * 256;  // kept entries a warp lists before their pixels are marked (16 bits each)
 constexpr int kWarpsPerSM = 16;       // resident warps per SM the register budget is sized for
 
 // One item's row: entry e's staged value at v4[e / 4] (padding slots NaN).
@@ -427,12 +439,92 @@ __device__ __forceinline__ void warp_totals(const float (&ss)[Sums<MODE>::NF], c
   unpack_totals<MODE>(th, tl, n_set, h, l);
 }
 
+// Class ends of a row, in groups of 4 entries (coefficient class c holds the
+// groups [end(c - 1), end(c))).
+struct ClassEnds {
+  int e0, e1, e2, e3;
+  __device__ __forceinline__ int end(int c) const { return c == 0 ? e0 : (c == 1 ? e1 : (c == 2 ? e2 : e3)); }
+};
+
+// Walk of a lane over its groups of every coefficient class in turn: from a
+// class's first group on, the lane takes every 32nd of its every step-th
+// groups, in blocks of kRing. quick(v, k, lo, c) gets group k of the block at
+// lo of class c where all lanes have the whole block and room() holds (the
+// same on all lanes), else fn(v, q, c) gets the lane's groups of the block
+// one after another. close(c) follows the last group of each class, empty
+// ones after the first group included.
+//
+// The groups come through the lane's own slots of a ring in shared memory, a
+// block ahead of their use whatever class they belong to (16-byte cp.async
+// copies; a lane reads only what it copied, so no barrier is needed): a
+// warp's loads stay in flight through the whole row. With register loads, a
+// block at a time and each class by itself, a warp waited for memory at every
+// block (3.2 of the 7.3 cycles an instruction).
+template <int NCLS, class R, class Q, class F, class C>
+__device__ __forceinline__ void stream_row(const Row& row, const ClassEnds& ge, int lane, int step, uint32_t ring,
+                                           R&& room, Q&& quick, F&& fn, C&& close) {
+  const int hop = 32 * step, mine = lane * step;
+  auto settle = [&](int& c, int& lo, int& hi) {   // to the next class with groups left
+    if (NCLS > 1) {
+      while (lo >= hi && c + 1 < NCLS) {
+        lo = hi;
+        ++c;
+        hi = ge.end(c);
+      }
+    }
+  };
+  int c = 0, lo = 0, hi = ge.e0;
+  settle(c, lo, hi);   // (leading empty classes have nothing to close: all sums are 0)
+  // copies of the block of kRing groups from `p` on, of which the lane has
+  // `left` groups of 32 step each to the class's end
+  auto issue = [&](const float4* p, int left) {
+#pragma unroll
+    for (int k = 0; k < kRing; ++k)
+      if (hop * k < left)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(ring + 512u * k), "l"(p + hop * k) : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  auto take = [&](int k) {   // group k of the block that has arrived
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(ring + 512u * k) : "memory");
+    return v;
+  };
+  issue(row.v4 + lo + mine, hi - lo - mine);
+#pragma unroll 1
+  while (lo < hi) {
+    int nc = c, nlo = lo + hop * kRing, nhi = hi;
+    settle(nc, nlo, nhi);
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (lo + hop * kRing <= hi && room()) {
+      float4 v[kRing];
+#pragma unroll
+      for (int k = 0; k < kRing; ++k) v[k] = take(k);
+      issue(row.v4 + nlo + mine, nhi - nlo - mine);   // under way while this block is used
+#pragma unroll
+      for (int k = 0; k < kRing; ++k) quick(v[k], k, lo, c);
+    } else {
+#pragma unroll 1
+      for (int k = 0; lo + hop * k < hi && k < kRing; ++k)
+        if (lo + hop * k + mine < hi) fn(take(k), lo + hop * k + mine, c);
+      issue(row.v4 + nlo + mine, nhi - nlo - mine);
+    }
+    for (const int stop = nlo < nhi ? nc : NCLS; c < stop; ++c) close(c);
+    c = nc;
+    lo = nlo;
+    hi = nhi;
+  }
+}
+
+// A coefficient class's weight (1, 3/4, 1/2, 1/4).
+__device__ __forceinline__ float class_weight(int c) { return 1.0f - 0.25f * (float)c; }
+
 // Pass A (one lane's share): plain FP32 sums about 0 of the finite entries
 // of every `step`-th group of 4 (a sample of a long row: they only place
 // the core), in the layout unpack_totals reads (per-lane values).
 template <int MODE>
-__device__ __forceinline__ void lane_full_sums(const Row& row, const float* wts, const int (&ge)[4],
-                                               int lane, int step, float (&ss)[Sums<MODE>::NF],
+__device__ __forceinline__ void lane_full_sums(const Row& row, const float* wts, const ClassEnds& ge,
+                                               int lane, int step, uint32_t ring, float (&ss)[Sums<MODE>::NF],
                                                uint32_t (&ci)[Sums<MODE>::NI]) {
   constexpr int NF = Sums<MODE>::NF, NI = Sums<MODE>::NI;
 #pragma unroll
@@ -440,43 +532,46 @@ __device__ __forceinline__ void lane_full_sums(const Row& row, const float* wts,
 #pragma unroll
   for (int i = 0; i < NI; ++i) ci[i] = 0u;
   if (MODE == MODE_CLASS || MODE == MODE_UNIT) {
-    constexpr int NCLS = MODE == MODE_CLASS ? 4 : 1;
-    int lo = 0;
-#pragma unroll 1
-    for (int cls = 0; cls < NCLS; ++cls) {
-      const int hi = ge[cls];
-      uint32_t cnt = 0;
-      float s1 = 0.0f, s2 = 0.0f;
-      scan_row(row, lo >> 2, hi >> 2, lane, [&](const float4& v4, int) {
-        const float xs[4] = {v4.x, v4.y, v4.z, v4.w};
+    uint32_t cnt = 0;
+    float s1 = 0.0f, s2 = 0.0f;
+    auto add = [&](const float4& v4) {
+      const float xs[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (fabsf(xs[j]) <= FLT_MAX) {   // finite (padding slots hold NaN)
-            ++cnt;
-            s1 = __fadd_rn(s1, xs[j]);
-            s2 = __fmaf_rn(xs[j], xs[j], s2);
-          }
-        }
-      }, step);
+      for (int j = 0; j < 4; ++j) {
+        // finite entries (padding slots hold NaN)
+        asm("{\n\t.reg .pred p;\n\t.reg .f32 m;\n\t"
+            "abs.f32 m, %3;\n\t"
+            "setp.le.f32 p, m, 0f7f7fffff;\n\t"
+            "@p add.u32 %0, %0, 1;\n\t"
+            "@p add.rn.f32 %1, %1, %3;\n\t"
+            "@p fma.rn.f32 %2, %3, %3, %2;\n\t}"
+            : "+r"(cnt), "+f"(s1), "+f"(s2) : "f"(xs[j]));
+      }
+    };
+    stream_row<MODE == MODE_CLASS ? 4 : 1>(
+        row, ge, lane, step, ring, [] { return true; }, [&](const float4& v4, int, int, int) { add(v4); },
+        [&](const float4& v4, int, int) { add(v4);
+    }, [&](int cls) {
       if (MODE == MODE_CLASS) {
-        const float w = 1.0f - 0.25f * (float)cls, w2 = w * w;
+        const float w = class_weight(cls), w2 = w * w;
         const uint32_t pk = cnt << (16 * (cls & 1));
         if (cls < 2) ci[0] += pk;
         else ci[NI - 1] += pk;
         ss[0] = fmaf(w, s1, ss[0]);
         ss[1] = fmaf(w2, s1, ss[1]);
         ss[2] = fmaf(w2, s2, ss[2]);
+        cnt = 0;
+        s1 = s2 = 0.0f;
       } else {
         ci[0] = cnt;
         ss[0] = s1;
         ss[1] = s2;
       }
-      lo = hi;
-    }
+    });
   } else {
     uint32_t cnt = 0;
     float om = 0.0f, a1 = 0.0f, oo = 0.0f, b1 = 0.0f, b2 = 0.0f;
-    scan_row(row, 0, ge[3] >> 2, lane, [&](const float4& v4, int q) {
+    scan_row(row, 0, ge.e3, lane, [&](const float4& v4, int q) {
       const float xs[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -499,14 +594,13 @@ __device__ __forceinline__ void lane_full_sums(const Row& row, const float* wts,
 
 // Pass B (one lane's share): sums about Kf of the entries inside
 // [cLo, cHi] (the layout unpack_totals reads); every other valid entry goes to the
-// lane's tail: slot k at tl[32 k] = (value bits, entry index | class <<
-// 16), written for every entry and kept only for the tail (m counts the
-// slots kept, so the branch-free store of a core entry is overwritten).
-// Returns false when a group of 4 entries found fewer than 4 of the tcap
-// slots left (the sums are then incomplete).
+// lane's tail: slot k at tl[32 k] = (value bits, entry index | the upper half
+// of its class weight's bits), m slots in all. Returns false when a group of
+// 4 entries found fewer than 4 of the tcap slots left (the sums are then
+// incomplete).
 template <int MODE, bool KAHAN>
-__device__ __forceinline__ bool lane_core_sums(const Row& row, const float* wts, const int (&ge)[4], int lane,
-                                               float cLo, float cHi, float Kf, uint2* tl, int tcap, int& m,
+__device__ __forceinline__ bool lane_core_sums(const Row& row, const float* wts, const ClassEnds& ge, int lane,
+                                               float cLo, float cHi, float Kf, uint2* tl, int tcap, uint32_t ring, int& m,
                                                float (&ss)[Sums<MODE>::NF], float (&cc)[Sums<MODE>::NF],
                                                uint32_t (&ci)[Sums<MODE>::NI]) {
   constexpr int NF = Sums<MODE>::NF, NI = Sums<MODE>::NI;
@@ -517,35 +611,69 @@ __device__ __forceinline__ bool lane_core_sums(const Row& row, const float* wts,
   m = 0;
   bool fit = true;
   if (MODE == MODE_CLASS || MODE == MODE_UNIT) {
-    constexpr int NCLS = MODE == MODE_CLASS ? 4 : 1;
-    int lo = 0;
-#pragma unroll 1
-    for (int cls = 0; cls < NCLS; ++cls) {
-      const int hi = ge[cls];
-      uint32_t cnt = 0;
-      Acc<KAHAN> a1, a2;
-      scan_row(row, lo >> 2, hi >> 2, lane, [&](const float4& v4, int q) {
-        if (m + 4 > tcap) fit = false;
-        if (!fit) return;
-        const float xs[4] = {v4.x, v4.y, v4.z, v4.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const bool core = xs[j] >= cLo && xs[j] <= cHi;
-          if (core) {
-            const float d = __fsub_rn(xs[j], Kf);
-            ++cnt;
-            a1.add(d);
-            a2.add_prod(d, d);
-          }
-          tl[32 * m] = make_uint2(__float_as_uint(xs[j]), (uint32_t)(4 * q + j) | ((uint32_t)cls << 16));
-          m += (!core && xs[j] == xs[j]) ? 1 : 0;
+    float cnt = 0.0f;   // (exact: a row holds fewer than 2^16 entries)
+    Acc<KAHAN> a1, a2;
+    uint32_t at = (uint32_t)__cvta_generic_to_shared(tl);      // the lane's next tail slot
+    const uint32_t at0 = at, most = at + 256u * (uint32_t)(tcap - 4);   // 4 slots left
+    // one entry: into the sums, or into the tail, or (NaN) neither
+    auto put = [&](float x, uint32_t tag) {
+      if (KAHAN) {
+        if (x >= cLo && x <= cHi) {
+          const float d = __fsub_rn(x, Kf);
+          cnt += 1.0f;
+          a1.add(d);
+          a2.add_prod(d, d);
+        } else if (x == x) {
+          asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at), "r"(__float_as_uint(x)), "r"(tag) : "memory");
+          at += 256u;
         }
-      });
-      if (!fit) return false;
+      } else {
+        // without a branch: most groups of a warp hold both kinds
+        asm volatile(
+            "{\n\t.reg .pred core, out;\n\t.reg .f32 d;\n\t"
+            "setp.ge.f32 core, %4, %6;\n\t"
+            "setp.le.and.f32 core, %4, %7, core;\n\t"
+            "setp.num.and.f32 out, %4, %4, !core;\n\t"
+            "sub.rn.f32 d, %4, %8;\n\t"
+            "@core add.rn.f32 %0, %0, d;\n\t"
+            "@core fma.rn.f32 %1, d, d, %1;\n\t"
+            "@core add.rn.f32 %2, %2, 0f3f800000;\n\t"
+            "@out st.shared.v2.b32 [%3], {%4, %5};\n\t"
+            "@out add.u32 %3, %3, 256;\n\t}"
+            : "+f"(a1.s), "+f"(a2.s), "+f"(cnt), "+r"(at)
+            : "f"(x), "r"(tag), "f"(cLo), "f"(cHi), "f"(Kf)
+            : "memory");
+      }
+    };
+    auto tag_of = [&](int q, int cls) {
+      return (uint32_t)(4 * q) | (MODE == MODE_CLASS ? __float_as_uint(class_weight(cls)) : 0u);
+    };
+    stream_row<MODE == MODE_CLASS ? 4 : 1>(
+        row, ge, lane, 1, ring,
+        // no lane can run out of slots within a block
+        [&] { return !__any_sync(0xffffffffu, (int32_t)(at + 256u * 4 * (kRing - 1) - most) > 0); },
+        [&](const float4& v4, int k, int lo, int cls) {
+          const uint32_t tag = tag_of(lo + lane, cls) + 128u * k;
+          put(v4.x, tag);
+          put(v4.y, tag + 1);
+          put(v4.z, tag + 2);
+          put(v4.w, tag + 3);
+        },
+        [&](const float4& v4, int q, int cls) {
+          if ((int32_t)(at - most) > 0) {
+            fit = false;
+          } else {
+            const uint32_t tag = tag_of(q, cls);
+            put(v4.x, tag);
+            put(v4.y, tag + 1);
+            put(v4.z, tag + 2);
+            put(v4.w, tag + 3);
+          }
+    }, [&](int cls) {
       const float s1 = a1.val(), s2 = a2.val();
       if (MODE == MODE_CLASS) {
-        const float w = 1.0f - 0.25f * (float)cls, w2 = w * w;
-        const uint32_t pk = cnt << (16 * (cls & 1));
+        const float w = class_weight(cls), w2 = w * w;
+        const uint32_t pk = (uint32_t)cnt << (16 * (cls & 1));
         if (cls < 2) ci[0] += pk;
         else ci[NI - 1] += pk;
         if (KAHAN) {
@@ -558,16 +686,20 @@ __device__ __forceinline__ bool lane_core_sums(const Row& row, const float* wts,
           ss[1] = fmaf(w2, s1, ss[1]);
           ss[2] = fmaf(w2, s2, ss[2]);
         }
+        cnt = 0.0f;
+        a1 = Acc<KAHAN>();
+        a2 = Acc<KAHAN>();
       } else {
-        ci[0] = cnt;
+        ci[0] = (uint32_t)cnt;
         ss[0] = a1.s; cc[0] = a1.c; ss[1] = a2.s; cc[1] = a2.c;
       }
-      lo = hi;
-    }
+    });
+    m = (int)((at - at0) >> 8);
+    if (!fit) return false;
   } else {
     uint32_t cnt = 0;
     Acc<KAHAN> om, a1, oo, b1, b2;
-    scan_row(row, 0, ge[3] >> 2, lane, [&](const float4& v4, int q) {
+    scan_row(row, 0, ge.e3, lane, [&](const float4& v4, int q) {
       if (m + 4 > tcap) fit = false;
       if (!fit) return;
       const float xs[4] = {v4.x, v4.y, v4.z, v4.w};
@@ -602,8 +734,8 @@ __device__ __forceinline__ bool lane_core_sums(const Row& row, const float* wts,
 // One lane's share of a full pass over [Ln, Hn] about Kf (the layout
 // unpack_totals reads), read from the staged row.
 template <int MODE, bool KAHAN>
-__device__ __noinline__ void lane_range_sums(const Row& row, const float* wts, const int (&ge)[4],
-                                                int lane, float Ln, float Hn, float Kf,
+__device__ __noinline__ void lane_range_sums(const Row& row, const float* wts, const ClassEnds& ge,
+                                                int lane, float Ln, float Hn, float Kf, uint32_t ring,
                                                 float (&ss)[Sums<MODE>::NF], float (&cc)[Sums<MODE>::NF],
                                                 uint32_t (&ci)[Sums<MODE>::NI]) {
   constexpr int NF = Sums<MODE>::NF, NI = Sums<MODE>::NI;
@@ -612,28 +744,39 @@ __device__ __noinline__ void lane_range_sums(const Row& row, const float* wts, c
 #pragma unroll
   for (int i = 0; i < NI; ++i) ci[i] = 0u;
   if (MODE == MODE_CLASS || MODE == MODE_UNIT) {
-    constexpr int NCLS = MODE == MODE_CLASS ? 4 : 1;
-    int lo = 0;
-#pragma unroll 1
-    for (int cls = 0; cls < NCLS; ++cls) {
-      const int hi = ge[cls];
-      uint32_t cnt = 0;
-      Acc<KAHAN> a1, a2;
-      scan_row(row, lo >> 2, hi >> 2, lane, [&](const float4& v4, int) {
-        const float xs[4] = {v4.x, v4.y, v4.z, v4.w};
+    uint32_t cnt = 0;
+    Acc<KAHAN> a1, a2;
+    auto add = [&](const float4& v4) {
+      const float xs[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+      for (int j = 0; j < 4; ++j) {
+        if (KAHAN) {
           if (xs[j] >= Ln && xs[j] <= Hn) {
             const float d = __fsub_rn(xs[j], Kf);
             ++cnt;
             a1.add(d);
             a2.add_prod(d, d);
           }
+        } else {
+          asm("{\n\t.reg .pred p;\n\t.reg .f32 d;\n\t"
+              "setp.ge.f32 p, %3, %4;\n\t"
+              "setp.le.and.f32 p, %3, %5, p;\n\t"
+              "sub.rn.f32 d, %3, %6;\n\t"
+              "@p add.u32 %0, %0, 1;\n\t"
+              "@p add.rn.f32 %1, %1, d;\n\t"
+              "@p fma.rn.f32 %2, d, d, %2;\n\t}"
+              : "+r"(cnt), "+f"(a1.s), "+f"(a2.s)
+              : "f"(xs[j]), "f"(Ln), "f"(Hn), "f"(Kf));
         }
-      });
+      }
+    };
+    stream_row<MODE == MODE_CLASS ? 4 : 1>(
+        row, ge, lane, 1, ring, [] { return true; }, [&](const float4& v4, int, int, int) { add(v4); },
+        [&](const float4& v4, int, int) { add(v4);
+    }, [&](int cls) {
       const float s1 = a1.val(), s2 = a2.val();
       if (MODE == MODE_CLASS) {
-        const float w = 1.0f - 0.25f * (float)cls, w2 = w * w;
+        const float w = class_weight(cls), w2 = w * w;
         const uint32_t pk = cnt << (16 * (cls & 1));
         if (cls < 2) ci[0] += pk;
         else ci[NI - 1] += pk;
@@ -647,16 +790,18 @@ __device__ __noinline__ void lane_range_sums(const Row& row, const float* wts, c
           ss[1] = fmaf(w2, s1, ss[1]);
           ss[2] = fmaf(w2, s2, ss[2]);
         }
+        cnt = 0;
+        a1 = Acc<KAHAN>();
+        a2 = Acc<KAHAN>();
       } else {
         ci[0] = cnt;
         ss[0] = a1.s; cc[0] = a1.c; ss[1] = a2.s; cc[1] = a2.c;
       }
-      lo = hi;
-    }
+    });
   } else {
     uint32_t cnt = 0;
     Acc<KAHAN> om, a1, oo, b1, b2;
-    scan_row(row, 0, ge[3] >> 2, lane, [&](const float4& v4, int q) {
+    scan_row(row, 0, ge.e3, lane, [&](const float4& v4, int q) {
       const float xs[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -681,36 +826,108 @@ __device__ __noinline__ void lane_range_sums(const Row& row, const float* wts, c
 }
 
 // One lane's tail entries inside [Ln, Hn]: (Omega, A1, OO, B1, B2) about Kf
-// and their count (m: the lane's slots).
+// and their count (m: the lane's slots). Four entries at a time, so their
+// reads are under way together.
 template <int MODE, bool KAHAN>
 __device__ __forceinline__ void lane_tail_sums(const uint2* tl, const float* wts, int m, float Ln, float Hn,
                                                float Kf, float (&ss)[5], float (&cc)[5], uint32_t& cnt) {
   Acc<KAHAN> acc[5];
   cnt = 0;
-  for (int k = 0; k < m; ++k) {
-    const uint2 t = tl[32 * k];
-    const float v = __uint_as_float(t.x);
-    if (v >= Ln && v <= Hn) {
-      float w;
-      if (MODE == MODE_CLASS) w = 1.0f - 0.25f * (float)(t.y >> 16);
-      else if (MODE == MODE_UNIT) w = 1.0f;
-      else w = wts[t.y & 0xffffu];
-      const float d = __fsub_rn(v, Kf);
-      const float w2 = __fmul_rn(w, w);
-      const float w2d = __fmul_rn(w2, d);
-      ++cnt;
-      acc[0].add(w);
-      acc[1].add(__fmul_rn(w, d));
-      acc[2].add(w2);
-      acc[3].add(w2d);
-      acc[4].add_prod(w2d, d);
+#pragma unroll 1
+  for (int k0 = 0; k0 < m; k0 += 4) {
+    uint2 t[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      t[u] = make_uint2(0x7fc00000u, 0u);   // NaN: in no interval
+      if (k0 + u < m) t[u] = tl[32 * (k0 + u)];
     }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float v = __uint_as_float(t[u].x);
+      const float w = MODE == MODE_CLASS ? __uint_as_float(t[u].y & 0xffff0000u)
+                                         : (MODE == MODE_UNIT ? 1.0f : wts[t[u].y & 0xffffu]);
+      if (KAHAN) {
+        if (v >= Ln && v <= Hn) {
+          const float d = __fsub_rn(v, Kf);
+          const float w2 = __fmul_rn(w, w);
+          const float w2d = __fmul_rn(w2, d);
+          ++cnt;
+          acc[0].add(w);
+          acc[1].add(__fmul_rn(w, d));
+          acc[2].add(w2);
+          acc[3].add(w2d);
+          acc[4].add_prod(w2d, d);
+        }
+      } else if (MODE == MODE_UNIT) {   // (unit weights: Omega = OO = count, B1 = A1)
+        asm("{\n\t.reg .pred p;\n\t.reg .f32 d;\n\t"
+            "setp.ge.f32 p, %3, %4;\n\t"
+            "setp.le.and.f32 p, %3, %5, p;\n\t"
+            "sub.rn.f32 d, %3, %6;\n\t"
+            "@p add.u32 %0, %0, 1;\n\t"
+            "@p add.rn.f32 %1, %1, d;\n\t"
+            "@p fma.rn.f32 %2, d, d, %2;\n\t}"
+            : "+r"(cnt), "+f"(acc[1].s), "+f"(acc[4].s)
+            : "f"(v), "f"(Ln), "f"(Hn), "f"(Kf));
+      } else {
+        asm("{\n\t.reg .pred p;\n\t.reg .f32 d, w2, wd, w2d;\n\t"
+            "setp.ge.f32 p, %6, %8;\n\t"
+            "setp.le.and.f32 p, %6, %9, p;\n\t"
+            "sub.rn.f32 d, %6, %10;\n\t"
+            "mul.rn.f32 w2, %7, %7;\n\t"
+            "mul.rn.f32 wd, %7, d;\n\t"
+            "mul.rn.f32 w2d, w2, d;\n\t"
+            "@p add.u32 %0, %0, 1;\n\t"
+            "@p add.rn.f32 %1, %1, %7;\n\t"
+            "@p add.rn.f32 %2, %2, wd;\n\t"
+            "@p add.rn.f32 %3, %3, w2;\n\t"
+            "@p add.rn.f32 %4, %4, w2d;\n\t"
+            "@p fma.rn.f32 %5, w2d, d, %5;\n\t}"
+            : "+r"(cnt), "+f"(acc[0].s), "+f"(acc[1].s), "+f"(acc[2].s), "+f"(acc[3].s), "+f"(acc[4].s)
+            : "f"(v), "f"(w), "f"(Ln), "f"(Hn), "f"(Kf));
+      }
+    }
+  }
+  if (!KAHAN && MODE == MODE_UNIT) {
+    acc[0].s = acc[2].s = (float)cnt;
+    acc[3].s = acc[1].s;
   }
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
     ss[v] = acc[v].s;
     cc[v] = acc[v].c;
   }
+}
+
+// Totals over the warp of the five tail sums (hi + lo, identical on every
+// lane). Sums of class weights and of their squares are multiples of 1/16
+// that binary32 holds exactly whatever their order: they travel as integers
+// (at most 177 entries a lane: 4 Omega below 2^15, 16 OO below 2^17), and
+// with unit weights they are the count.
+template <int MODE, int PREC>
+__device__ __forceinline__ void tail_totals(const float (&ts)[5], const float (&tc)[5], uint32_t count, float (&th)[5],
+                                            float (&tl)[5]) {
+  if (MODE == MODE_ENTRY) {
+    warp_sum<5, PREC>(ts, tc, th, tl);
+    return;
+  }
+  if (MODE == MODE_UNIT) {
+    th[0] = th[2] = (float)count;
+  } else {
+    const uint32_t mine = (uint32_t)(4.0f * ts[0]) + ((uint32_t)(16.0f * ts[2]) << 15);
+    const uint32_t all = __reduce_add_sync(0xffffffffu, mine);
+    th[0] = 0.25f * (float)(all & 0x7fffu);
+    th[2] = 0.0625f * (float)(all >> 15);
+  }
+  tl[0] = tl[2] = 0.0f;
+  constexpr int N = MODE == MODE_UNIT ? 2 : 3;
+  float s[N], c[N], h[N], l[N];
+  s[0] = ts[1]; c[0] = tc[1];
+  s[1] = ts[4]; c[1] = tc[4];
+  if (N > 2) { s[N - 1] = ts[3]; c[N - 1] = tc[3]; }
+  warp_sum<N, PREC>(s, c, h, l);
+  th[1] = h[0]; tl[1] = l[0];
+  th[4] = h[1]; tl[4] = l[1];
+  th[3] = h[N > 2 ? N - 1 : 0]; tl[3] = l[N > 2 ? N - 1 : 0];
 }
 
 // (h, l) += (a, b) for pairs, in the arithmetic of the precision mode.
@@ -752,10 +969,10 @@ __device__ __forceinline__ int sketch_element(int s, int G) {
 }
 
 template <int MODE>
-__device__ __forceinline__ void sample_features(const Row& row, const float* wts, const int (&ge)[4], int lane,
+__device__ __forceinline__ void sample_features(const Row& row, const float* wts, const ClassEnds& ge, int lane,
                                                 int step, float n_s, float om_s, float m1, float s1,
                                                 float (&feat)[kIn]) {
-  const int G = ge[3] >> 2;
+  const int G = ge.e3;
   // element s = 32 r + lane of the sketch in x[r] (+inf where none)
   float x[4];
 #pragma unroll
@@ -849,6 +1066,14 @@ __device__ __forceinline__ void mark_pixel(uint32_t* bm, const int32_t* cpix, in
   if (i >= 0) atomicOr(bm + (i >> 5), 1u << (i & 31));
 }
 
+// Marks the kept entries of a group (out of line: few groups hold one).
+__device__ __noinline__ void mark_group(uint32_t* bm, const int32_t* cpix, float4 v4, float thr, int64_t e) {
+  const float xs[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (xs[j] > thr) mark_pixel(bm, cpix, e + j);
+}
+
 // The first clip interval [lo, hi] from plain FP32 totals of the full set
 // about 0 (h: Omega, A1, OO, B1, B2; the formulas of finalise, poisson_sd
 // and clip_step in single rounding); only the core is placed with it.
@@ -885,15 +1110,20 @@ __global__ void __launch_bounds__(32 * kWarps, kWarpsPerSM / kWarps) k_clip_warp
   constexpr int NF = Sums<MODE>::NF, NI = Sums<MODE>::NI;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // [weights (MODE_ENTRY), shared by the warps] then per warp its tail
-  // (8-byte slots, slot k of lane l at 32 k + l)
+  // [weights (MODE_ENTRY), shared by the warps, or a ring of kRing groups a
+  // lane for each warp] then per warp its tail (8-byte slots, slot k of lane
+  // l at 32 k + l)
   const int capr = MODE == MODE_ENTRY ? (a.cap + 3) & ~3 : 0;
   float* wts = reinterpret_cast<float*>(smem_raw);
-  uint2* tail = reinterpret_cast<uint2*>(wts + capr) + (size_t)warp * (32 * a.tcap) + lane;
+  constexpr int kRingFloats = MODE == MODE_ENTRY ? 0 : kWarps * kRing * 128;
+  const uint32_t ring = (uint32_t)__cvta_generic_to_shared(smem_raw) + 4u * capr + (uint32_t)(warp * kRing * 512) +
+                        16u * lane;
+  uint2* tails = reinterpret_cast<uint2*>(wts + capr + kRingFloats);
+  uint2* tail = tails + (size_t)warp * (32 * a.tcap) + lane;
   // with inference (SURR 2) the network's normalisation and BF16 weights
   // follow the tails, copied once per CTA (read by every item, they would
   // otherwise compete with the streamed rows for the L1 cache)
-  float* nm_s = reinterpret_cast<float*>(reinterpret_cast<uint2*>(wts + capr) + (size_t)kWarps * 32 * a.tcap);
+  float* nm_s = reinterpret_cast<float*>(tails + (size_t)kWarps * 32 * a.tcap);
   __nv_bfloat16* w_s = reinterpret_cast<__nv_bfloat16*>(nm_s + kNNorm);
   (void)w_s;
   if (SURR == 2) {
@@ -933,9 +1163,9 @@ __global__ void __launch_bounds__(32 * kWarps, kWarpsPerSM / kWarps) k_clip_warp
     const int r0 = __ldg(a.rowptr + b);
     const int n = __ldg(a.rowptr + b + 1) - r0;      // multiple of 4
     const int nq = n >> 2;
-    int ge[4];   // end of coefficient class 0..3 in the row; weight-0 carriers follow
-#pragma unroll
-    for (int c = 0; c < 4; ++c) ge[c] = __ldg(a.grp + 4 * b + c);
+    // coefficient classes of the row; weight-0 carriers follow the last
+    const int4 g4 = __ldg(reinterpret_cast<const int4*>(a.grp) + b);
+    const ClassEnds ge{g4.x >> 2, g4.y >> 2, g4.z >> 2, g4.w >> 2};
 
     if (MODE == MODE_ENTRY) {
       for (int e = threadIdx.x; e < n; e += 32 * kWarps) {
@@ -961,7 +1191,7 @@ __global__ void __launch_bounds__(32 * kWarps, kWarpsPerSM / kWarps) k_clip_warp
         // (rows of 2048 entries and more: every 4th group of 4, 512 and more:
         // every 2nd)
         const int step = nq >= 512 ? 4 : (nq >= 128 ? 2 : 1);
-        lane_full_sums<MODE>(row, wts, ge, lane, step, ss, ci);
+        lane_full_sums<MODE>(row, wts, ge, lane, step, ring, ss, ci);
 #pragma unroll
         for (int v = 0; v < NF; ++v) cz[v] = 0.0f;
         float n_set, h[6], l[6], lo, hi, mu, sd;
@@ -1011,7 +1241,7 @@ __global__ void __launch_bounds__(32 * kWarps, kWarpsPerSM / kWarps) k_clip_warp
           float ss[NF], cc[NF];
           uint32_t ci[NI];
           const bool fit =
-              lane_core_sums<MODE, KAHAN>(row, wts, ge, lane, cLo, cHi, K, tail, a.tcap, m, ss, cc, ci);
+              lane_core_sums<MODE, KAHAN>(row, wts, ge, lane, cLo, cHi, K, tail, a.tcap, ring, m, ss, cc, ci);
           ovf = __any_sync(0xffffffffu, !fit);
           ++scans;
           if (a.clip_stats) {
@@ -1042,24 +1272,28 @@ __global__ void __launch_bounds__(32 * kWarps, kWarpsPerSM / kWarps) k_clip_warp
           float ts[5], tc[5], th[5], tl[5];
           uint32_t tn;
           lane_tail_sums<MODE, KAHAN>(tail, wts, m, Ln, Hn, K, ts, tc, tn);
-          warp_sum<5, TPREC>(ts, tc, th, tl);
           tn = __reduce_add_sync(0xffffffffu, tn);
           stat(3, 1);
-#pragma unroll
-          for (int v = 0; v < 5; ++v) {
-            h[v] = ch[v];
-            l[v] = cl[v];
-            add_pair<PREC>(h[v], l[v], th[v], tl[v]);
-          }
-          h[5] = l[5] = 0.0f;
           n_set = cn + (float)tn;
+#pragma unroll
+          for (int v = 0; v < 6; ++v) h[v] = l[v] = 0.0f;
+          if (st.steps < 0 || n_set != st.n_cur) {   // (an unchanged set ends the loop with the moments it has)
+            tail_totals<MODE, TPREC>(ts, tc, tn, th, tl);
+#pragma unroll
+            for (int v = 0; v < 5; ++v) {
+              h[v] = ch[v];
+              l[v] = cl[v];
+              if (MODE != MODE_ENTRY && (v == 0 || v == 2)) h[v] = __fadd_rn(h[v], th[v]);   // exact
+              else add_pair<PREC>(h[v], l[v], th[v], tl[v]);
+            }
+          }
           Kf = K;
         } else {
           // a tail overflowed: a full pass over [Ln, Hn]
           float ss[NF], cc[NF];
           uint32_t ci[NI];
           Kf = st.Kf;
-          lane_range_sums<MODE, KAHAN>(row, wts, ge, lane, Ln, Hn, Kf, ss, cc, ci);
+          lane_range_sums<MODE, KAHAN>(row, wts, ge, lane, Ln, Hn, Kf, ring, ss, cc, ci);
           stat(6, 1);
           warp_totals<MODE, PREC>(ss, cc, ci, n_set, h, l);
         }
@@ -1103,18 +1337,68 @@ __global__ void __launch_bounds__(32 * kWarps, kWarpsPerSM / kWarps) k_clip_warp
         // without an overflow and with thr at or above the core, no core entry
         // exceeds thr: the lane's tail, then the weight-0 carriers of the row;
         // else every entry (padding slots hold NaN, never above a threshold)
-        const bool from_tail = MODE != MODE_ENTRY && !ovf && thr >= cHi;
-        if (from_tail) {
-          stat(5, 1);
-          for (int k = 0; k < m; ++k)
-            if (__uint_as_float(tail[32 * k].x) > thr) mark_pixel(bm, cp, (int64_t)(tail[32 * k].y & 0xffffu));
-        }
-        scan_row(row, from_tail ? ge[3] >> 2 : 0, nq, lane, [&](const float4& v4, int q) {
-          const float xs[4] = {v4.x, v4.y, v4.z, v4.w};
+        if (MODE == MODE_ENTRY) {   // (no ring to list in: each lane marks its own)
+          scan_row(row, 0, nq, lane, [&](const float4& v4, int q) {
+            if (fmaxf(fmaxf(v4.x, v4.y), fmaxf(v4.z, v4.w)) > thr) mark_group(bm, cp, v4, thr, 4 * q);
+          });
+        } else {
+          const bool from_tail = !ovf && thr >= cHi;
+          if (from_tail) stat(5, 1);
+          // The warp's kept entries are listed first (by ballots, in the idle
+          // ring), then looked up a lane each, so the pixel loads of an item's
+          // kept pixels are in flight together: with each lane looking up its
+          // own, a warp waited for memory once a slot or two, a quarter of the
+          // kernel's time.
+          uint16_t* lst = reinterpret_cast<uint16_t*>(smem_raw) + warp * kMarkList;
+          const uint32_t below = (1u << lane) - 1u;
+          const int most = from_tail ? (int)__reduce_max_sync(0xffffffffu, m) : 0;
+          int k = 0, q = from_tail ? ge.e3 : 0;
+          while (k < most || q < nq) {
+            int listed = 0;
+#pragma unroll 1
+            for (; k < most && listed <= kMarkList - 32; ++k) {
+              uint2 t = make_uint2(0x7fc00000u, 0u);
+              if (k < m) t = tail[32 * k];
+              const bool kept = __uint_as_float(t.x) > thr;
+              const uint32_t who = __ballot_sync(0xffffffffu, kept);
+              if (kept) lst[listed + __popc(who & below)] = (uint16_t)t.y;
+              listed += __popc(who);
+            }
+            if (k >= most) {
+#pragma unroll 1
+              for (; q < nq && listed <= kMarkList - 256; q += 64) {   // two groups a lane at a time
+                float4 v[2];
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (xs[j] > thr) mark_pixel(bm, cp, 4 * q + j);
-        });
+                for (int u = 0; u < 2; ++u) {
+                  const float nan = __int_as_float(0x7fc00000);
+                  v[u] = make_float4(nan, nan, nan, nan);
+                  if (q + 32 * u + lane < nq) v[u] = __ldg(row.v4 + q + 32 * u + lane);
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                  const float xs[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+                  for (int j = 0; j < 4; ++j) {
+                    const uint32_t who = __ballot_sync(0xffffffffu, xs[j] > thr);
+                    if (xs[j] > thr) lst[listed + __popc(who & below)] = (uint16_t)(4 * (q + 32 * u + lane) + j);
+                    listed += __popc(who);
+                  }
+                }
+              }
+            }
+            __syncwarp();
+#pragma unroll 1
+            for (int i = lane; i < listed; i += 128) {
+              int32_t px[4];
+#pragma unroll
+              for (int u = 0; u < 4; ++u) px[u] = i + 32 * u < listed ? __ldg(cp + lst[i + 32 * u]) : -1;
+#pragma unroll
+              for (int u = 0; u < 4; ++u)
+                if (px[u] >= 0) atomicOr(bm + (px[u] >> 5), 1u << (px[u] & 31));
+            }
+            __syncwarp();
+          }
+        }
       }
       __syncwarp();   // the tail is rewritten by the warp's next frame
     }
@@ -1154,19 +1438,32 @@ int sm_count() {
   return cached[dev];
 }
 
+// Shared memory of the surrogate's network in an inference launch.
+constexpr long kNetBytes = kNNorm * 4 + ((kNParams * 2 + 15) & ~15);
+
+// Tail slots a lane has. When its slots run out an item's remaining steps run
+// as full passes, whose sums round differently, so the number is part of the
+// results: it follows from the longest row and the plan's block size alone
+// (what 1/12 of the row needs, at most what a block of that size had room for
+// with a row's entry weights beside the tails), not from the launch's layout.
+long clip_tail_cap(bool weights, int32_t cap, int warps, int surr) {
+  const long wbytes = weights ? 4 * (((long)cap + 3) & ~3L) : 0;
+  const long budget = (long)smem_optin() - kClipStaticSmem - wbytes - (surr == 2 ? kNetBytes : 0);
+  long tcap = clip_tail_slots(cap, 32 * warps);
+  if (warps * 256 * tcap > budget) tcap = std::max(0L, budget / (256L * warps));
+  return tcap < 5 ? 0 : tcap;   // (no room for a tail: every step runs as a full pass)
+}
+
+// Shared memory of a launch: a row's weights or the warps' rings, and the tails.
+size_t clip_launch_bytes(bool weights, int32_t cap, int warps, long tcap, int surr) {
+  const long head = weights ? 4 * (((long)cap + 3) & ~3L) : (long)warps * kRing * 512;
+  return (size_t)(head + warps * 256 * tcap + (surr == 2 ? kNetBytes : 0));
+}
+
 template <int MODE, int PREC, int kWarps, int SURR>
-cudaError_t launch_warp_t(ClipArgs a, int n_ctas, int mode, cudaStream_t s) {
-  // shared memory: the weights of a row (per-entry weights only), then
-  // each warp's tail (8 bytes a slot, 32 lanes)
-  const long capr = ((long)a.cap + 3) & ~3L;
-  const long wbytes = MODE == MODE_ENTRY ? 4 * capr : 0;
-  const long budget = (long)smem_optin() - kClipStaticSmem - wbytes -
-                     (SURR == 2 ? kNNorm * 4 + ((kNParams * 2 + 15) & ~15) : 0);
-  long tcap = clip_tail_slots(a.cap, 32 * kWarps);
-  if (kWarps * 256 * tcap > budget) tcap = std::max(0L, budget / (256L * kWarps));
-  if (tcap < 5) tcap = 0;   // no room for a tail: every step runs as a full pass
+cudaError_t launch_warp_t(ClipArgs a, int n_ctas, long tcap, int mode, cudaStream_t s) {
   a.tcap = (int32_t)tcap;
-  const size_t smem = (size_t)(wbytes + kWarps * 256 * tcap + (SURR == 2 ? kNNorm * 4 + ((kNParams * 2 + 15) & ~15) : 0));
+  const size_t smem = clip_launch_bytes(MODE == MODE_ENTRY, a.cap, kWarps, tcap, SURR);
   auto k = k_clip_warp<MODE, PREC, kWarps, SURR>;
   // resident CTAs per multiprocessor of this instance at this shared-memory
   // size, cached per device (the first query comes before any capture: the
@@ -1223,11 +1520,16 @@ cudaError_t launch_warp_t(ClipArgs a, int n_ctas, int mode, cudaStream_t s) {
 
 template <int MODE, int PREC, int SURR = 0>
 cudaError_t launch_tail_b(const ClipArgs& a, int n_ctas, int tpb, int mode, cudaStream_t s) {
-  switch (tpb) {
-    case 32: return launch_warp_t<MODE, PREC, 1, SURR>(a, n_ctas, mode, s);
-    case 64: return launch_warp_t<MODE, PREC, 2, SURR>(a, n_ctas, mode, s);
-    case 128: return launch_warp_t<MODE, PREC, 4, SURR>(a, n_ctas, mode, s);
-    default: return launch_warp_t<MODE, PREC, 8, SURR>(a, n_ctas, mode, s);
+  int warps = tpb == 32 || tpb == 64 || tpb == 128 ? tpb / 32 : 8;
+  const long tcap = clip_tail_cap(MODE == MODE_ENTRY, a.cap, warps, SURR);
+  // the widest block up to the plan's whose rings and tails fit
+  while (warps > 1 && clip_launch_bytes(MODE == MODE_ENTRY, a.cap, warps, tcap, SURR) + kClipStaticSmem > (size_t)smem_optin())
+    warps /= 2;
+  switch (warps) {
+    case 1: return launch_warp_t<MODE, PREC, 1, SURR>(a, n_ctas, tcap, mode, s);
+    case 2: return launch_warp_t<MODE, PREC, 2, SURR>(a, n_ctas, tcap, mode, s);
+    case 4: return launch_warp_t<MODE, PREC, 4, SURR>(a, n_ctas, tcap, mode, s);
+    default: return launch_warp_t<MODE, PREC, 8, SURR>(a, n_ctas, tcap, mode, s);
   }
 }
 
