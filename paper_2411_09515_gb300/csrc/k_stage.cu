@@ -4,16 +4,32 @@
 // e's value, padding slots NaN), so the clip kernel reads each bin's values
 // as one contiguous run.
 //
-// One CTA per image tile (kTileH x kTileW pixels) and group of frames.
-// Threads read tile rows: each thread four consecutive pixels (one vector
-// load where the row is aligned), two frames per step (four in the ring
-// kernel); the corrected tile sits in shared memory by pixel, then the
-// tile's list of (slot, pixel) pairs, ascending by slot, writes it out (the
-// entries of one bin inside a tile occupy consecutive slots). Each value is
-// the same IEEE sequence as pixel_value(): RN32(RN32(adc - pedestal) /
-// gain), then RN32(. / norm).
+// One CTA per image tile (kTileH x kTileW pixels) and group of frames, four
+// frames a step: each thread corrects four consecutive pixels of a tile row
+// in the four frames and stores a pixel's four values side by side in shared
+// memory; then the tile's list of (slot, pixel) pairs, ascending by slot,
+// writes them out (the entries of one bin inside a tile occupy consecutive
+// slots), one 16-byte read and four stores a slot. The tile is double
+// buffered, so a step costs one barrier and the warps of a CTA correct the
+// next frames while others still write the last. The raw words of later
+// frames arrive meanwhile in a ring in shared memory (cp.async into the
+// thread's own slots: no registers held, no barrier).
+//
+// Each value is the same IEEE sequence as pixel_value(): RN32(RN32(adc -
+// pedestal) / gain), then RN32(. / norm); level 0 without a division (Level0).
+//
+// What bounds it: the staged values written (27 MB a Jungfrau-4M frame, all
+// of whole sectors) and the words read. With one value a shared-memory access
+// and range tests a pixel and frame, the kernel was bound by its instructions
+// and shared-memory wavefronts: 48 raw Jungfrau-4M frames 475 -> 411 us (4.6
+// TB/s); the write-out is half of it. Float frames that had no ring (a width
+// that is not a multiple of 4, or a list of frames): 29 frames of 1031 x 1065
+// 80 -> 75 us; 24 frames of 619 x 487, whose 80 CTAs left half of the GPU
+// idle: 60 -> 26 us.
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "sep_device.cuh"
 #include "sep_internal.h"
@@ -22,331 +38,255 @@ namespace sep {
 namespace {
 
 constexpr int kTilePix = kTileH * kTileW;
-constexpr int kTileSlots = kTilePix + 4;   // the tile's values, then a NaN (padding slots read it)
 constexpr int kStageThreads = kTilePix / 4;   // 4 consecutive pixels of one row a thread
 constexpr int kRowThreads = kTileW / 4;       // threads covering one tile row
+constexpr int kStep = 4;                      // frames a step
 static_assert(kTileW % 4 == 0 && kStageThreads % 32 == 0 && kStageThreads <= 1024, "tile shape");
 
-// Four consecutive raw words / values of one frame (VEC: one aligned vector load).
-template <int DT, bool VEC>
-__device__ __forceinline__ void load4(const void* frame, int64_t p, bool (&in)[4], uint32_t (&w)[4]) {
-  if (DT == SEP_DTYPE_U16_JF) {
-    const uint16_t* f = reinterpret_cast<const uint16_t*>(frame);
-    if (VEC) {
-      const uint2 v = __ldg(reinterpret_cast<const uint2*>(f + p));
-      w[0] = v.x & 0xffffu; w[1] = v.x >> 16; w[2] = v.y & 0xffffu; w[3] = v.y >> 16;
-    } else {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) w[k] = in[k] ? __ldg(f + p + k) : 0u;
-    }
-  } else {
-    const float* f = reinterpret_cast<const float*>(frame);
-    if (VEC) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(f + p));
-      w[0] = __float_as_uint(v.x); w[1] = __float_as_uint(v.y); w[2] = __float_as_uint(v.z); w[3] = __float_as_uint(v.w);
-    } else {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) w[k] = in[k] ? __float_as_uint(__ldg(f + p + k)) : 0u;
-    }
-  }
+// How a thread's four words of a frame reach the ring: one copy (columns a
+// multiple of 4, aligned frames), copies of 4 bytes (aligned to those), or
+// not at all (plain loads: raw frames of an odd width or address).
+enum { LOAD_VECTOR = 2, LOAD_WORD = 1, LOAD_PLAIN = 0 };
+
+// Frames the ring holds (what shared memory allows beside the two tiles).
+template <int DT>
+__host__ __device__ constexpr int ring_frames() {
+  return DT == SEP_DTYPE_U16_JF ? 8 : 4;
+}
+template <int DT, int LOAD>
+constexpr size_t stage_smem_bytes() {
+  return sizeof(float4) * 2 * (kTilePix + 1) +
+         (LOAD == LOAD_PLAIN ? 0 : (size_t)ring_frames<DT>() * kStageThreads * (DT == SEP_DTYPE_U16_JF ? 8 : 16));
 }
 
-// The tile's (slot, shared-memory index) pairs a thread writes: pairs tid +
-// kStageThreads k for k < kScReg stay in registers for every frame, longer
-// lists read the rest at each scatter. Padding pairs point at the NaN.
+// The tile's pairs a thread writes: pairs tid + kStageThreads k for
+// k < kScReg stay in registers for every frame, longer lists read the rest at
+// each step (with 7 instead of 8 a 512-frame Jungfrau-4M batch takes 13.3
+// instead of 12.4 ms: its tiles near the beam hold up to 8,000 pairs). loc: the pixel's place in the tile, four consecutive pixels
+// kStageThreads apart (the threads of a warp then store side by side);
+// kTilePix, a NaN, for padding.
 constexpr int kScReg = 8;
+__device__ __forceinline__ int tile_place(int pix) {
+  return pix < 0 ? kTilePix : (pix & 3) * kStageThreads + (pix >> 2);
+}
 
-struct TileScatter {
-  int slot[kScReg], loc[kScReg];
-  int n;   // pairs held
-  __device__ __forceinline__ void load(const StageArgs& a, int eb, int ne) {
-    n = 0;
-#pragma unroll
-    for (int k = 0; k < kScReg; ++k) {
-      const int j = threadIdx.x + kStageThreads * k;
-      int2 sc = make_int2(0, kTilePix);
-      if (j < ne) {
-        sc = __ldg(a.tile_sc + eb + j);
-        n = k + 1;
-      }
-      slot[k] = sc.x;
-      loc[k] = sc.y >= 0 ? sc.y : kTilePix;
-    }
+template <int DT, bool NORM, int LOAD>
+__global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
+  constexpr int kWord = DT == SEP_DTYPE_U16_JF ? 2 : 4;
+  constexpr int kRing = ring_frames<DT>();
+  extern __shared__ __align__(16) unsigned char stage_smem[];
+  float4* tv = reinterpret_cast<float4*>(stage_smem);   // [2][kTilePix + 1]: a pixel's values of the step's frames
+  unsigned char* ring = stage_smem + sizeof(float4) * 2 * (kTilePix + 1);
+  const int t = blockIdx.x;
+  const int tid = threadIdx.x;
+  const int eb = __ldg(a.tile_ebase + t), ne = __ldg(a.tile_ebase + t + 1) - eb;
+  if (ne == 0) return;
+  if (tid < 2) {
+    const float nan = __int_as_float(0x7fc00000);
+    tv[tid * (kTilePix + 1) + kTilePix] = make_float4(nan, nan, nan, nan);
   }
-};
-
-// Scatter of NF corrected tiles (tv[h]) of frames f .. f + NF - 1 (the
-// first nf of them) to their entries' slots.
-template <int NF>
-__device__ __forceinline__ void scatter_tile(const StageArgs& a, const TileScatter& ts, const float (*tv)[kTileSlots],
-                                             int eb, int ne, int64_t f, int nf) {
-  float* out[NF];
-#pragma unroll
-  for (int h = 0; h < NF; ++h) out[h] = a.stage + (f + min(h, nf - 1)) * a.npos;
+  uint32_t slot[kScReg];   // the pairs' slots and places
+  int loc[kScReg];
 #pragma unroll
   for (int k = 0; k < kScReg; ++k) {
-    if (k >= ts.n) break;
-#pragma unroll
-    for (int h = 0; h < NF; ++h)
-      if (h < nf) out[h][ts.slot[k]] = tv[h][ts.loc[k]];
+    int2 sc = make_int2(0, -1);
+    if (tid + kStageThreads * k < ne) sc = __ldg(a.tile_sc + eb + tid + kStageThreads * k);
+    slot[k] = (uint32_t)sc.x;
+    loc[k] = tile_place(sc.y);
   }
-  for (int j = threadIdx.x + kStageThreads * kScReg; j < ne; j += kStageThreads) {
-    const int2 sc = __ldg(a.tile_sc + eb + j);
-    const int l = sc.y >= 0 ? sc.y : kTilePix;
-#pragma unroll
-    for (int h = 0; h < NF; ++h)
-      if (h < nf) out[h][sc.x] = tv[h][l];
-  }
-}
-
-template <int DT, bool NORM, bool VEC>
-__global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
-  __shared__ float tv[2][kTileSlots];
-  const int t = blockIdx.x;
-  const int tid = threadIdx.x;
-  const int eb = __ldg(a.tile_ebase + t), ne = __ldg(a.tile_ebase + t + 1) - eb;
-  if (ne == 0) return;
-  if (tid < 2) tv[tid][kTilePix] = __int_as_float(0x7fc00000);
-  TileScatter ts;
-  ts.load(a, eb, ne);
-  const int loc0 = (tid / kRowThreads) * kTileW + 4 * (tid % kRowThreads);   // this thread's pixels in the tile
   const int64_t r = (int64_t)(t / a.tiles_x) * kTileH + tid / kRowThreads;
   const int64_t c = (int64_t)(t % a.tiles_x) * kTileW + 4 * (tid % kRowThreads);
   const int64_t p = r * a.cols + c;    // first of this thread's 4 pixels
-  bool in[4];
-  float p0[4], g0[4], nm[4];
-  bool any = false;
+  const int n_in = r < a.rows ? (int)max((int64_t)0, min((int64_t)4, a.cols - c)) : 0;   // of them inside the image
+  Level0 cal[4];
+  float nm[4];
+  bool usual = true;   // level-0 words of these pixels need no division
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    in[k] = r < a.rows && c + k < a.cols;
-    any = any || in[k];
-    p0[k] = 0.0f;
-    g0[k] = 1.0f;
     nm[k] = 1.0f;
-    if (in[k]) {
+    if (k < n_in) {
       if (DT == SEP_DTYPE_U16_JF) {
-        p0[k] = __ldg(a.ped + p + k);
-        g0[k] = __ldg(a.gain + p + k);
+        cal[k].set(__ldg(a.ped + p + k), __ldg(a.gain + p + k));
+        usual = usual && cal[k].limit != 0;
       }
       if (NORM) nm[k] = __ldg(a.norm + p + k);
     }
-  }
-  const int f0 = blockIdx.y * a.frames_per_cta;
-  const int f1 = min(f0 + a.frames_per_cta, a.n_frames);
-  // two frames per step: both frames' loads are in flight together
-  for (int f = f0; f < f1; f += 2) {
-    const int nf = min(2, f1 - f);
-    uint32_t w[2][4];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (h < nf && any) {
-        const void* frame = a.fptr ? (const void*)a.fptr[f + h] : frame_ptr<DT>(a.frames, f + h, a.npix);
-        load4<DT, VEC>(frame, p, in, w[h]);
-      }
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (h >= nf) continue;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (!in[k]) continue;
-        float x;
-        if (DT == SEP_DTYPE_U16_JF) {
-          const uint32_t u = w[h][k], code = u >> 14;
-          float ped = p0[k], gain = g0[k];
-          if (code != 0) {   // gain levels 1 and 2
-            const int64_t lvl = code == 1 ? 1 : 2;
-            ped = __ldg(a.ped + lvl * a.npix + p + k);
-            gain = __ldg(a.gain + lvl * a.npix + p + k);
-          }
-          x = __fdiv_rn(__fsub_rn((float)(u & 0x3FFFu), ped), gain);
-        } else {
-          x = __uint_as_float(w[h][k]);
-        }
-        if (NORM) x = __fdiv_rn(x, nm[k]);
-        tv[h][loc0 + k] = x;
-      }
-    }
-    __syncthreads();
-    scatter_tile<2>(a, ts, tv, eb, ne, f, nf);
-    __syncthreads();
-  }
-}
-
-// The aligned case with the frames' loads ahead of their use: each thread
-// copies its four raw words (8 bytes; 16 for FP32 input) of the next frames
-// into its own slots of a ring in shared memory (cp.async, no registers
-// held), kRing frames ahead, and reads them back when their frame comes.
-// A thread reads only what it copied itself, so the ring needs no barrier.
-// Four frames per step share the two barriers around the write-out.
-constexpr int kRing = 8;   // frames ahead (a multiple of the 4 frames of a step)
-
-// Dynamic shared memory of k_stage_ring: four corrected tiles, then the ring.
-template <int DT>
-constexpr size_t ring_smem_bytes() {
-  return sizeof(float) * 4 * kTileSlots + (size_t)kRing * kStageThreads * (DT == SEP_DTYPE_U16_JF ? 8 : 16);
-}
-
-template <int DT, bool NORM>
-__global__ void __launch_bounds__(kStageThreads) k_stage_ring(StageArgs a) {
-  constexpr int kVec = DT == SEP_DTYPE_U16_JF ? 8 : 16;   // bytes of 4 raw words
-  extern __shared__ __align__(16) unsigned char stage_smem[];
-  float(*tv)[kTileSlots] = reinterpret_cast<float(*)[kTileSlots]>(stage_smem);
-  unsigned char(*ring)[kStageThreads * kVec] =
-      reinterpret_cast<unsigned char(*)[kStageThreads * kVec]>(stage_smem + sizeof(float) * 4 * kTileSlots);
-  const int t = blockIdx.x;
-  const int tid = threadIdx.x;
-  const int eb = __ldg(a.tile_ebase + t), ne = __ldg(a.tile_ebase + t + 1) - eb;
-  if (ne == 0) return;
-  if (tid < 4) tv[tid][kTilePix] = __int_as_float(0x7fc00000);
-  TileScatter ts;
-  ts.load(a, eb, ne);
-  const int loc0 = (tid / kRowThreads) * kTileW + 4 * (tid % kRowThreads);   // this thread's pixels in the tile
-  const int64_t r = (int64_t)(t / a.tiles_x) * kTileH + tid / kRowThreads;
-  const int64_t c = (int64_t)(t % a.tiles_x) * kTileW + 4 * (tid % kRowThreads);
-  const int64_t p = r * a.cols + c;    // first of this thread's 4 pixels
-  // (columns are a multiple of 4: a thread's 4 pixels are all inside or all outside)
-  const bool inside = r < a.rows && c < a.cols;
-  float p0[4], g0[4], r0[4], nm[4];
-  const bool any = inside;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    p0[k] = 0.0f;
-    g0[k] = 1.0f;
-    nm[k] = 1.0f;
-    if (inside) {
-      if (DT == SEP_DTYPE_U16_JF) {
-        p0[k] = __ldg(a.ped + p + k);
-        g0[k] = __ldg(a.gain + p + k);
-      }
-      if (NORM) nm[k] = __ldg(a.norm + p + k);
-    }
-    // level-0 reciprocal for the division below; 0 (= use the IEEE
-    // division) outside the range where the correction step is exact
-    const float ag = fabsf(g0[k]);
-    r0[k] = ag >= 0x1p-100f && ag <= 0x1p100f ? __frcp_rn(g0[k]) : 0.0f;
   }
   const int f0 = blockIdx.y * a.frames_per_cta;
   const int nfr = min(f0 + a.frames_per_cta, a.n_frames) - f0;
-  const unsigned slot0 = (unsigned)__cvta_generic_to_shared(&ring[0][tid * kVec]);
-  // one commit group per frame (empty past the last frame or for idle threads)
-  auto issue = [&](int j) {
-    if (any && j < nfr) {
-      const char* src = reinterpret_cast<const char*>(frame_ptr<DT>(a.frames, f0 + j, a.npix)) +
-                        p * (DT == SEP_DTYPE_U16_JF ? 2 : 4);
-      const unsigned dst = slot0 + (unsigned)((j % kRing) * kStageThreads * kVec);
-      if (kVec == 8)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
-      else
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+  const int64_t pitch = a.npix * kWord;   // bytes from a frame to the next
+  const unsigned char* first = reinterpret_cast<const unsigned char*>(frame_ptr<DT>(a.frames, f0, a.npix)) + p * kWord;
+  auto frame_of = [&](int j) {   // this thread's first word of frame f0 + j
+    return a.fptr ? reinterpret_cast<const unsigned char*>((uintptr_t)a.fptr[f0 + j]) + p * kWord : first + j * pitch;
+  };
+  const unsigned ring0 = (unsigned)__cvta_generic_to_shared(ring) + tid * 4 * kWord;
+  // copy of a frame's words from src to ring slot q
+  auto copy = [&](int q, const unsigned char* src) {
+    const unsigned dst = ring0 + (unsigned)(q * kStageThreads * 4 * kWord);
+    if (LOAD == LOAD_VECTOR) {
+      if (kWord == 2) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
+      else asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+    } else {
+      // (raw: the width is even, so a pair of pixels is inside or outside)
+#pragma unroll
+      for (int k = 0; k < 4; k += 4 / kWord)
+        if (k < n_in)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst + k * kWord), "l"(src + k * kWord)
+                       : "memory");
+    }
+  };
+  // the step's frames from j0 on into the ring slots from q0 on (one commit
+  // group a step, empty past the last frame)
+  auto issue = [&](int j0, int q0) {
+    if (n_in > 0) {
+#pragma unroll
+      for (int h = 0; h < kStep; ++h)
+        if (j0 + h < nfr) copy(q0 + h, frame_of(j0 + h));
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
   };
+  if (LOAD != LOAD_PLAIN) {
 #pragma unroll
-  for (int j = 0; j < kRing; ++j) issue(j);
-  for (int j = 0; j < nfr; j += 4) {
-    const int nf = min(4, nfr - j);
-    // groups 0 .. j + kRing - 1 issued: frames j .. j + 3 have landed
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(kRing - 4) : "memory");
-    uint32_t w[4][4];
+    for (int j = 0; j < kRing; j += kStep) issue(j, j);
+  }
+  int buf = 0;
+  for (int j = 0; j < nfr; j += kStep, buf ^= 1) {
+    const int nf = min(kStep, nfr - j);
+    const int q0 = j % kRing;   // ring slots of the step's frames
+    float4* tile = tv + buf * (kTilePix + 1);
+    float x[kStep][4];
+    bool rest = !usual;   // another gain level, or an unusual calibration
+    if (DT == SEP_DTYPE_U16_JF) {
+      uint2 v[kStep];   // a frame's four words
+      if (LOAD != LOAD_PLAIN) {
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(kRing / kStep - 1) : "memory");
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const unsigned char* sl = &ring[(j + h) % kRing][tid * kVec];
-      if (DT == SEP_DTYPE_U16_JF) {
-        const uint2 v = *reinterpret_cast<const uint2*>(sl);
-        w[h][0] = v.x & 0xffffu; w[h][1] = v.x >> 16; w[h][2] = v.y & 0xffffu; w[h][3] = v.y >> 16;
+        for (int h = 0; h < kStep; ++h)
+          v[h] = *reinterpret_cast<const uint2*>(ring + ((q0 + h) * kStageThreads + tid) * 8);
       } else {
-        const uint4 v = *reinterpret_cast<const uint4*>(sl);
-        w[h][0] = v.x; w[h][1] = v.y; w[h][2] = v.z; w[h][3] = v.w;
-      }
-    }
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      if (h >= nf) continue;
+        for (int h = 0; h < kStep; ++h) {
+          const uint16_t* src = reinterpret_cast<const uint16_t*>(h < nf ? frame_of(j + h) : nullptr);
+          uint32_t w[4];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (!inside) continue;
-        float x;
-        if (DT == SEP_DTYPE_U16_JF) {
-          const uint32_t u = w[h][k], code = u >> 14;
-          const float d0 = __fsub_rn((float)(u & 0x3FFFu), p0[k]);
-          const float q0 = __fmul_rn(d0, r0[k]);
-          const float aq = fabsf(q0);
-          if (code == 0 && r0[k] != 0.0f && ((aq >= 0x1p-125f && aq <= 0x1p125f) || d0 == 0.0f)) {
-            // RN((adc - ped) / gain) without a division: with r = RN(1/gain)
-            // and q = RN(d r), the residual e = d - q gain is exact under a
-            // fused multiply-add, and RN(q + e r) is the correctly rounded
-            // quotient (Markstein's correction, IBM J. Res. Dev. 34(1), 1990);
-            // the range tests keep gain, quotient and residual normal,
-            // elsewhere the IEEE division runs
-            x = __fmaf_rn(__fmaf_rn(-q0, g0[k], d0), r0[k], q0);
-          } else {
-            float ped = p0[k], gain = g0[k];
-            if (code != 0) {   // gain levels 1 and 2
-              const int64_t lvl = code == 1 ? 1 : 2;
-              ped = __ldg(a.ped + lvl * a.npix + p + k);
-              gain = __ldg(a.gain + lvl * a.npix + p + k);
-            }
-            x = __fdiv_rn(__fsub_rn((float)(u & 0x3FFFu), ped), gain);
-          }
-        } else {
-          x = __uint_as_float(w[h][k]);
+          for (int k = 0; k < 4; ++k) w[k] = h < nf && k < n_in ? (uint32_t)__ldg(src + k) : 0u;
+          v[h] = make_uint2(w[0] | w[1] << 16, w[2] | w[3] << 16);
         }
-        if (NORM) x = __fdiv_rn(x, nm[k]);
-        tv[h][loc0 + k] = x;
+      }
+      uint32_t all = 0;
+#pragma unroll
+      for (int h = 0; h < kStep; ++h) {
+        all |= v[h].x | v[h].y;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          // the word's value as a float without a conversion: its 16 bits
+          // below the exponent of 2^23, less 2^23 (exact)
+          const uint32_t bits = __byte_perm(k < 2 ? v[h].x : v[h].y, 0x4b000000u, k & 1 ? 0x7432 : 0x7410);
+          x[h][k] = cal[k].value_of(__fsub_rn(__uint_as_float(bits), 8388608.0f));
+          if (NORM) x[h][k] = __fdiv_rn(x[h][k], nm[k]);
+        }
+      }
+      rest = rest || (all & 0xc000c000u);
+    } else {
+      if (LOAD != LOAD_PLAIN) asm volatile("cp.async.wait_group %0;\n" ::"n"(kRing / kStep - 1) : "memory");
+#pragma unroll
+      for (int h = 0; h < kStep; ++h) {
+        const float4 v = *reinterpret_cast<const float4*>(ring + ((q0 + h) * kStageThreads + tid) * 16);
+        x[h][0] = v.x; x[h][1] = v.y; x[h][2] = v.z; x[h][3] = v.w;
+        if (NORM) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) x[h][k] = __fdiv_rn(x[h][k], nm[k]);
+        }
       }
     }
-    // the slots just read are refilled (this thread's own words, already in registers)
-    issue(j + kRing);
-    issue(j + kRing + 1);
-    issue(j + kRing + 2);
-    issue(j + kRing + 3);
+    // the slots just read are refilled (this thread's own words, in registers now)
+    if (LOAD != LOAD_PLAIN) issue(j + kRing, q0);
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      tile[k * kStageThreads + tid] = make_float4(x[0][k], x[1][k], x[2][k], x[3][k]);
+    if (DT == SEP_DTYPE_U16_JF && rest && n_in > 0) {
+      for (int h = 0; h < nf; ++h) {   // (rare: one copy of the code)
+        const void* fr = a.fptr ? (const void*)a.fptr[f0 + j + h] : frame_ptr<DT>(a.frames, f0 + j + h, a.npix);
+        for (int k = 0; k < n_in; ++k)
+          reinterpret_cast<float*>(tile + k * kStageThreads + tid)[h] =
+              pixel_value<DT, NORM>(fr, p + k, a.npix, a.ped, a.gain, a.norm);
+      }
+    }
     __syncthreads();
-    scatter_tile<4>(a, ts, tv, eb, ne, (int64_t)(f0 + j), nf);
-    __syncthreads();
+    // the step's frames, slot by slot
+    float* out = a.stage + (int64_t)(f0 + j) * a.npos;
+    if (nf == kStep) {
+      float *o1 = out + a.npos, *o2 = o1 + a.npos, *o3 = o2 + a.npos;
+      auto put = [&](uint32_t q, const float4& v) {
+        out[q] = v.x;
+        o1[q] = v.y;
+        o2[q] = v.z;
+        o3[q] = v.w;
+      };
+#pragma unroll
+      for (int k = 0; k < kScReg; ++k)
+        if (tid + kStageThreads * k < ne) put(slot[k], tile[loc[k]]);
+      for (int q = tid + kStageThreads * kScReg; q < ne; q += kStageThreads) {
+        const int2 sc = __ldg(a.tile_sc + eb + q);
+        put((uint32_t)sc.x, tile[tile_place(sc.y)]);
+      }
+    } else {   // the last step of a group: one copy of the code
+#pragma unroll 1
+      for (int q = tid; q < ne; q += kStageThreads) {
+        const int2 sc = __ldg(a.tile_sc + eb + q);
+        const float4 v = tile[tile_place(sc.y)];
+        float* o = out + (uint32_t)sc.x;
+        *o = v.x;
+        if (nf > 1) o[a.npos] = v.y;
+        if (nf > 2) o[2 * a.npos] = v.z;
+      }
+    }
   }
 }
 
-template <int DT, bool NORM>
-cudaError_t launch_v(const StageArgs& a, dim3 grid, bool vec, cudaStream_t s) {
-  if (vec) {
-    constexpr size_t smem = ring_smem_bytes<DT>();
-    if (smem > 48 * 1024) {
-      // opt in once per device (the attribute only needs to be set before
-      // the first launch; later calls find it set)
-      static bool set[64] = {};
-      int dev = 0;
-      if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
-      if (!set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(k_stage_ring<DT, NORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-        set[dev] = true;
-      }
-    }
-    k_stage_ring<DT, NORM><<<grid, kStageThreads, smem, s>>>(a);
-  } else {
-    k_stage<DT, NORM, false><<<grid, kStageThreads, 0, s>>>(a);
+template <int DT, bool NORM, int LOAD>
+cudaError_t launch_l(const StageArgs& a, dim3 grid, cudaStream_t s) {
+  constexpr size_t smem = stage_smem_bytes<DT, LOAD>();
+  // opt in once per device (the attribute only needs to be set before the
+  // first launch; later calls find it set)
+  static bool set[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = 0;
+  if (!set[dev]) {
+    cudaError_t e =
+        cudaFuncSetAttribute(k_stage<DT, NORM, LOAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    set[dev] = true;
   }
+  k_stage<DT, NORM, LOAD><<<grid, kStageThreads, smem, s>>>(a);
   return cudaGetLastError();
+}
+
+template <int DT, bool NORM>
+cudaError_t launch_v(const StageArgs& a, dim3 grid, cudaStream_t s) {
+  // One copy of a thread's four words: every frame at an address aligned to
+  // them and the rows' pixels in groups of 4. Copies of 4 bytes: float frames
+  // (their words), raw frames of an even width at 4-byte addresses.
+  if (a.align % (DT == SEP_DTYPE_U16_JF ? 8 : 16) == 0 && a.cols % 4 == 0) return launch_l<DT, NORM, LOAD_VECTOR>(a, grid, s);
+  if (DT == SEP_DTYPE_F32 || (a.align % 4 == 0 && a.cols % 2 == 0)) return launch_l<DT, NORM, LOAD_WORD>(a, grid, s);
+  return launch_l<DT, NORM, LOAD_PLAIN>(a, grid, s);
 }
 
 }  // namespace
 
-cudaError_t launch_stage(const StageArgs& a, int32_t dtype, bool has_norm, cudaStream_t s) {
-  if (a.n_frames <= 0) return cudaSuccess;
+cudaError_t launch_stage(const StageArgs& args, int32_t dtype, bool has_norm, cudaStream_t s) {
+  if (args.n_frames <= 0) return cudaSuccess;
+  StageArgs a = args;
   const int n_tiles = a.tiles_x * a.tiles_y;
+  // Frames a CTA: 32, which read the tile's calibration and list once for
+  // all, fewer (whole steps) where the grid would hold less than four CTAs a
+  // multiprocessor.
+  const int64_t share = (int64_t)n_tiles * a.n_frames / (152 * 4) / kStep * kStep;
+  a.frames_per_cta = (int)std::min<int64_t>(std::max<int64_t>(share, kStep), 32);
   dim3 grid(n_tiles, (a.n_frames + a.frames_per_cta - 1) / a.frames_per_cta);
-  // vector loads need every thread's 4 pixels aligned: a column count that
-  // is a multiple of 4 (tiles start at multiples of 128), frames contiguous
-  // or listed at 16-byte aligned addresses
-  bool vec = a.cols % 4 == 0;
-  if (!a.fptr) vec = vec && ((uintptr_t)a.frames % 16 == 0);
   if (dtype == SEP_DTYPE_U16_JF)
-    return has_norm ? launch_v<SEP_DTYPE_U16_JF, true>(a, grid, vec && !a.fptr, s)
-                    : launch_v<SEP_DTYPE_U16_JF, false>(a, grid, vec && !a.fptr, s);
-  return has_norm ? launch_v<SEP_DTYPE_F32, true>(a, grid, vec && !a.fptr, s)
-                  : launch_v<SEP_DTYPE_F32, false>(a, grid, vec && !a.fptr, s);
+    return has_norm ? launch_v<SEP_DTYPE_U16_JF, true>(a, grid, s) : launch_v<SEP_DTYPE_U16_JF, false>(a, grid, s);
+  return has_norm ? launch_v<SEP_DTYPE_F32, true>(a, grid, s) : launch_v<SEP_DTYPE_F32, false>(a, grid, s);
 }
 
 }  // namespace sep

@@ -282,9 +282,10 @@ sep::ClipArgs clip_args(sep_ctx* ctx, const sep_csr* csr, const float* stage, in
 }
 
 // Correction + staging of n frames (contiguous at `frames`, or listed in
-// fptr) into stage [n][stage_stride].
+// fptr, their addresses or-ed in fptr_align) into stage [n][stage_stride].
 cudaError_t enqueue_stage(sep_ctx* ctx, const sep_csr* csr, const sep_calib* calib, const void* frames,
-                          const uint64_t* fptr, int32_t dtype, int32_t n, float* stage, cudaStream_t s) {
+                          const uint64_t* fptr, int32_t dtype, int32_t n, float* stage, cudaStream_t s,
+                          uint64_t fptr_align = 1) {
   sep::StageArgs g;
   g.frames = frames;
   g.fptr = fptr;
@@ -295,7 +296,8 @@ cudaError_t enqueue_stage(sep_ctx* ctx, const sep_csr* csr, const sep_calib* cal
   g.tiles_x = csr->h.tiles_x;
   g.tiles_y = csr->h.tiles_y;
   g.n_frames = n;
-  g.frames_per_cta = std::min(n, 32);   // calibration and ranks are read once per CTA
+  // (contiguous frames: the first one's address and their pitch)
+  g.align = fptr ? fptr_align : (uint64_t)(uintptr_t)frames | (uint64_t)csr->npix * (dtype == SEP_DTYPE_U16_JF ? 2 : 4);
   g.ped = calib && dtype == SEP_DTYPE_U16_JF ? calib->d_ped : nullptr;
   g.gain = calib && dtype == SEP_DTYPE_U16_JF ? calib->d_gain : nullptr;
   g.norm = csr->d_norm;
@@ -1365,7 +1367,9 @@ sep_status sep_process_mixed(sep_ctx* ctx, int32_t n_det, sep_csr* const* csrs, 
       pa.npos = stage_stride(csr);
       set_interp(pa, csr, params);
       if (e == cudaSuccess) e = cudaMemsetAsync(bm, 0, (size_t)(words[d] * m) * 4, sd);
-      if (e == cudaSuccess) e = enqueue_stage(ctx, csr, calib, nullptr, fptr, dtype, m, stage, sd);
+      uint64_t align = 0;
+      for (int32_t g : members[d]) align |= (uint64_t)(uintptr_t)frames[g].frame_dev;
+      if (e == cudaSuccess) e = enqueue_stage(ctx, csr, calib, nullptr, fptr, dtype, m, stage, sd, align);
       if (e == cudaSuccess) e = enqueue_clip(ctx, csr, ca, params->precision, mode, sd, false);
       if (e == cudaSuccess && params->interpolate)
         e = sep::launch_mark_interp(pa, m, csr->h.nbins, mean_dev, sigma_dev, params->k_pick, bm, words[d], sd);

@@ -55,8 +55,9 @@ struct Level0 {
     const float ag = fabsf(g), ap = fabsf(p);
     limit = ag >= 0x1p-40f && ag <= 0x1p40f && (p == 0.0f || (ap >= 0x1p-60f && ap <= 0x1p60f)) ? 0x4000u : 0u;
   }
-  __device__ __forceinline__ float value(uint32_t u) const {
-    const float d = __fsub_rn((float)u, ped);
+  __device__ __forceinline__ float value(uint32_t u) const { return value_of((float)u); }
+  __device__ __forceinline__ float value_of(float adc) const {
+    const float d = __fsub_rn(adc, ped);
     const float q = __fmul_rn(d, r);
     return __fmaf_rn(__fmaf_rn(-q, gain, d), r, q);
   }

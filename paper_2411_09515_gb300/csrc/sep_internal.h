@@ -145,7 +145,8 @@ struct StageArgs {         // correction + staging of a batch (k_stage)
   const uint64_t* fptr;    // per frame address (mixed batches), may be null
   int64_t npix, npos;      // npos: the staged row stride (slots, >= nnz)
   int32_t rows, cols, tiles_x, tiles_y;
-  int32_t n_frames, frames_per_cta;
+  int32_t n_frames, frames_per_cta = 0;   // (frames a CTA: set at launch)
+  uint64_t align = 0;      // the bits of all the frames' addresses, or-ed: their common alignment
   const float* ped;        // [3][npix] (raw input)
   const float* gain;       // [3][npix]
   const float* norm;       // [npix] or null
