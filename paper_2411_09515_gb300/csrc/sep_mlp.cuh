@@ -72,7 +72,7 @@ cudaError_t launch_mlp_grad(const __nv_bfloat16* wbf, const float* x, const floa
 cudaError_t launch_adam(float* theta, __nv_bfloat16* wbf, __nv_bfloat16* wbt, float* m, float* v, float* grad, float lr,
                         int64_t step, cudaStream_t s);
 cudaError_t launch_mlp_forward(const __nv_bfloat16* wbf, const float* x, int64_t n, float* y, cudaStream_t s);
-cudaError_t launch_zero(float* p, int64_t n, cudaStream_t s);
+cudaError_t launch_zero(float* p, int64_t n, cudaStream_t s, float* q = nullptr);   // p[0 .. n), and *q with q
 int64_t prep_blocks(int64_t n);
 cudaError_t launch_prep_stats(const float* f, const float* t, int64_t n, int32_t* cnt, double* part, cudaStream_t s);
 cudaError_t launch_prep_scatter(const float* f, const float* t, int64_t n, const int64_t* base, const float* norm,

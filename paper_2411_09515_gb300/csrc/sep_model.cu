@@ -158,8 +158,7 @@ sep_status sep_mlp_loss_grad(sep_model* m, const float* x_dev, const float* t_de
   if (!m || n < 1 || !x_dev || !t_dev || !grad_dev || !loss_dev) return SEP_ERR_ARG;
   MCUDA(m->ctx, cudaSetDevice(m->ctx->device));
   cudaStream_t s = (cudaStream_t)stream;
-  MCUDA(m->ctx, sep::launch_zero(grad_dev, sep::kNParams, s));
-  MCUDA(m->ctx, sep::launch_zero(loss_dev, 1, s));
+  MCUDA(m->ctx, sep::launch_zero(grad_dev, sep::kNParams, s, loss_dev));
   MCUDA(m->ctx, sep::launch_mlp_grad(m->d_wbf, x_dev, t_dev, n, n, 0, 1, grad_dev, loss_dev, s));
   return SEP_OK;
 }
