@@ -23,10 +23,13 @@
 
 namespace {
 
-constexpr size_t kNoallocScratchBytes = (size_t)16 << 20;   // 16 MiB
+constexpr size_t kNoallocScratchBytes = (size_t)16 << 20;   // 16 MiB: what a batch may ask for
+// A batch asks for a tile count per 8192 bitmap words; the compaction's tiles
+// are smaller, at most 4 bytes more per 2048 words and frame, which this holds.
+constexpr size_t kNoallocExtraBytes = (size_t)64 << 10;
 constexpr int kMaxDevices = 64;
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes + kNoallocExtraBytes];
 
 // Device address of g_noalloc_scratch for each device (a host variable named
 // g_noalloc_scratch is only a host-side stand-in, never a device address).
@@ -63,9 +66,10 @@ extern "C" sep_status sep_sparsify_noalloc(sep_ctx* ctx, const sep_csr* csr, con
   words = (words + 7) & ~(int64_t)7;
   const size_t bm_bytes = align256((size_t)(words * n_frames) * 4);
   const size_t thr_bytes = align256((size_t)n_frames * (size_t)csr->h.nbins * 4);
-  const size_t aux_bytes = align256((size_t)sep::consumer_scratch_words(n_frames, words, 0) * 4);
+  const size_t aux_bytes = align256((size_t)n_frames * (size_t)((words + 8191) / 8192) * 4);
   const size_t need = bm_bytes + thr_bytes + aux_bytes;
-  if (need > kNoallocScratchBytes)
+  const size_t aux_used = align256((size_t)sep::consumer_scratch_words(n_frames, words, 0) * 4);
+  if (need > kNoallocScratchBytes || bm_bytes + thr_bytes + aux_used > sizeof(g_noalloc_scratch))
     return fail(SEP_ERR_ARG, "batch needs " + std::to_string(need) + " bytes of scratch; the static array holds " +
                                  std::to_string(kNoallocScratchBytes) + " (use fewer frames per call)");
 
