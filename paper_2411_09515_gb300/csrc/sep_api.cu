@@ -994,9 +994,16 @@ sep_status sep_process_host(sep_ctx* ctx, const sep_csr* csr, const sep_calib* c
                        (kept_capacity > 0 && (!idx_host || !val_host)) || (peak_capacity > 0 && !peaks_host)))
     return fail(ctx, SEP_ERR_ARG, "NULL argument");
   if (n_frames == 0) return SEP_OK;
-  const int32_t C = std::min(n_frames, chunk_frames > 0 ? chunk_frames : 64);
   const int64_t B = csr->h.nbins, N = csr->npix;
   const size_t px = dtype == SEP_DTYPE_U16_JF ? 2 : 4;
+  // Default chunks: 64 frames, which keep the kernels full, down to a quarter
+  // of a smaller batch, so that its copies overlap its kernels (16 raw
+  // Jungfrau-4M frames as one chunk wait for the whole copy-in before the
+  // first kernel and for the last one before the copy-out), but 32 MB of
+  // frames at least: below that a chunk's launches cost more than they hide.
+  const int64_t quarter = (n_frames + 3) / 4, least = ((int64_t)32 << 20) / (int64_t)(px * N) + 1;
+  const int32_t C = std::min(n_frames, chunk_frames > 0 ? chunk_frames
+                                                        : (int32_t)std::min<int64_t>(std::max(quarter, least), 64));
   // one slot: frames, mean, sigma, count, idx, val, n_kept, peaks, n_peaks (256-byte aligned pieces)
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t sz[9] = {al(px * N * C), al(4 * B * C), al(4 * B * C), al(4 * B * C), al(4 * kept_capacity * C),
