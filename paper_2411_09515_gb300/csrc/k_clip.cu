@@ -357,6 +357,7 @@ __device__ __forceinline__ void unpack_totals(const float* th, const float* tl, 
 // (other frames of the same bin) meet only between units of work.
 constexpr float kCoreMargin = 1.0f;   // core margin inside the clip interval, in deviations
 constexpr int kLoadsAhead = 4;        // 16-byte loads in flight per lane in a scan of the row
+constexpr int kPairsAhead = 2;        // the same for a value and its weight
 constexpr int kRing = 4;              // groups under way per lane in a walk of the row
 constexpr int kMarkList = kRing * 256;  // kept entries a warp lists before their pixels are marked (16 bits each)
 constexpr int kWarpsPerSM = 16;       // resident warps per SM the register budget is sized for
@@ -380,6 +381,32 @@ __device__ __forceinline__ void scan_row(const Row& row, int q0, int q1, int lan
 #pragma unroll
     for (int k = 0; k < kLoadsAhead; ++k)
       if (q + 32 * step * k < q1) fn(v[k], q + 32 * step * k);
+  }
+}
+
+// The same with the groups' entry weights: fn(v, w, q). The weights come
+// through the read-only path like the values (every frame of the bin reads
+// them, so all but the first reads hit the L2 or L1), two pairs at a time (three
+// spill). Held in shared memory beside the tails they left room for 5 to 7
+// warps on an SM; now 16 run: 1M pixels, 67 frames, norm, KAHAN 3046 -> 1560
+// us; a ragged detector with area fractions, 131 frames, 604 -> 423 us (whole
+// calls).
+template <class F>
+__device__ __forceinline__ void scan_weighted(const Row& row, const float* wts, int q0, int q1, int lane, F&& fn,
+                                              int step = 1) {
+  const float4* w4 = reinterpret_cast<const float4*>(wts);
+  for (int q = q0 + lane * step; q < q1; q += 32 * step * kPairsAhead) {
+    float4 v[kPairsAhead], w[kPairsAhead];
+#pragma unroll
+    for (int k = 0; k < kPairsAhead; ++k) {
+      if (q + 32 * step * k < q1) {
+        v[k] = __ldg(row.v4 + q + 32 * step * k);
+        w[k] = __ldg(w4 + q + 32 * step * k);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < kPairsAhead; ++k)
+      if (q + 32 * step * k < q1) fn(v[k], w[k], q + 32 * step * k);
   }
 }
 
@@ -571,11 +598,11 @@ __device__ __forceinline__ void lane_full_sums(const Row& row, const float* wts,
   } else {
     uint32_t cnt = 0;
     float om = 0.0f, a1 = 0.0f, oo = 0.0f, b1 = 0.0f, b2 = 0.0f;
-    scan_row(row, 0, ge.e3, lane, [&](const float4& v4, int q) {
-      const float xs[4] = {v4.x, v4.y, v4.z, v4.w};
+    scan_weighted(row, wts, 0, ge.e3, lane, [&](const float4& v4, const float4& w4, int) {
+      const float xs[4] = {v4.x, v4.y, v4.z, v4.w}, ws[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float w = wts[4 * q + j];
+        const float w = ws[j];
         if (w != 0.0f && fabsf(xs[j]) <= FLT_MAX) {
           const float w2 = __fmul_rn(w, w), w2d = __fmul_rn(w2, xs[j]);
           ++cnt;
@@ -595,7 +622,8 @@ __device__ __forceinline__ void lane_full_sums(const Row& row, const float* wts,
 // Pass B (one lane's share): sums about Kf of the entries inside
 // [cLo, cHi] (the layout unpack_totals reads); every other valid entry goes to the
 // lane's tail: slot k at tl[32 k] = (value bits, entry index | the upper half
-// of its class weight's bits), m slots in all. Returns false when a group of
+// of its class weight's bits, or with entry weights the weight's bits), m
+// slots in all. Returns false when a group of
 // 4 entries found fewer than 4 of the tcap slots left (the sums are then
 // incomplete).
 template <int MODE, bool KAHAN>
@@ -699,13 +727,13 @@ __device__ __forceinline__ bool lane_core_sums(const Row& row, const float* wts,
   } else {
     uint32_t cnt = 0;
     Acc<KAHAN> om, a1, oo, b1, b2;
-    scan_row(row, 0, ge.e3, lane, [&](const float4& v4, int q) {
+    scan_weighted(row, wts, 0, ge.e3, lane, [&](const float4& v4, const float4& w4, int) {
       if (m + 4 > tcap) fit = false;
       if (!fit) return;
-      const float xs[4] = {v4.x, v4.y, v4.z, v4.w};
+      const float xs[4] = {v4.x, v4.y, v4.z, v4.w}, ws[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float w = wts[4 * q + j];
+        const float w = ws[j];
         if (w == 0.0f) continue;
         if (xs[j] >= cLo && xs[j] <= cHi) {
           const float d = __fsub_rn(xs[j], Kf);
@@ -718,7 +746,7 @@ __device__ __forceinline__ bool lane_core_sums(const Row& row, const float* wts,
           b1.add(w2d);
           b2.add_prod(w2d, d);
         } else if (xs[j] == xs[j]) {
-          tl[32 * m] = make_uint2(__float_as_uint(xs[j]), (uint32_t)(4 * q + j));
+          tl[32 * m] = make_uint2(__float_as_uint(xs[j]), __float_as_uint(w));
           ++m;
         }
       }
@@ -801,11 +829,11 @@ __device__ __noinline__ void lane_range_sums(const Row& row, const float* wts, c
   } else {
     uint32_t cnt = 0;
     Acc<KAHAN> om, a1, oo, b1, b2;
-    scan_row(row, 0, ge.e3, lane, [&](const float4& v4, int q) {
-      const float xs[4] = {v4.x, v4.y, v4.z, v4.w};
+    scan_weighted(row, wts, 0, ge.e3, lane, [&](const float4& v4, const float4& w4, int) {
+      const float xs[4] = {v4.x, v4.y, v4.z, v4.w}, ws[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float w = wts[4 * q + j];
+        const float w = ws[j];
         if (w != 0.0f && xs[j] >= Ln && xs[j] <= Hn) {
           const float d = __fsub_rn(xs[j], Kf);
           const float w2 = __fmul_rn(w, w);
@@ -829,7 +857,7 @@ __device__ __noinline__ void lane_range_sums(const Row& row, const float* wts, c
 // and their count (m: the lane's slots). Four entries at a time, so their
 // reads are under way together.
 template <int MODE, bool KAHAN>
-__device__ __forceinline__ void lane_tail_sums(const uint2* tl, const float* wts, int m, float Ln, float Hn,
+__device__ __forceinline__ void lane_tail_sums(const uint2* tl, int m, float Ln, float Hn,
                                                float Kf, float (&ss)[5], float (&cc)[5], uint32_t& cnt) {
   Acc<KAHAN> acc[5];
   cnt = 0;
@@ -845,7 +873,7 @@ __device__ __forceinline__ void lane_tail_sums(const uint2* tl, const float* wts
     for (int u = 0; u < 4; ++u) {
       const float v = __uint_as_float(t[u].x);
       const float w = MODE == MODE_CLASS ? __uint_as_float(t[u].y & 0xffff0000u)
-                                         : (MODE == MODE_UNIT ? 1.0f : wts[t[u].y & 0xffffu]);
+                                         : (MODE == MODE_UNIT ? 1.0f : __uint_as_float(t[u].y));
       if (KAHAN) {
         if (v >= Ln && v <= Hn) {
           const float d = __fsub_rn(v, Kf);
@@ -982,7 +1010,7 @@ __device__ __forceinline__ void sample_features(const Row& row, const float* wts
     if (e >= 0) {
       const float4 q = __ldg(row.v4 + (e >> 2));
       const float c = (e & 3) == 0 ? q.x : ((e & 3) == 1 ? q.y : ((e & 3) == 2 ? q.z : q.w));
-      const bool ok = fabsf(c) <= FLT_MAX && (MODE != MODE_ENTRY || wts[e] != 0.0f);
+      const bool ok = fabsf(c) <= FLT_MAX && (MODE != MODE_ENTRY || __ldg(wts + e) != 0.0f);
       v = ok ? c : INFINITY;
     }
     x[r] = v;
@@ -1110,15 +1138,11 @@ __global__ void __launch_bounds__(32 * kWarps, kWarpsPerSM / kWarps) k_clip_warp
   constexpr int NF = Sums<MODE>::NF, NI = Sums<MODE>::NI;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // [weights (MODE_ENTRY), shared by the warps, or a ring of kRing groups a
-  // lane for each warp] then per warp its tail (8-byte slots, slot k of lane
-  // l at 32 k + l)
-  const int capr = MODE == MODE_ENTRY ? (a.cap + 3) & ~3 : 0;
-  float* wts = reinterpret_cast<float*>(smem_raw);
-  constexpr int kRingFloats = MODE == MODE_ENTRY ? 0 : kWarps * kRing * 128;
-  const uint32_t ring = (uint32_t)__cvta_generic_to_shared(smem_raw) + 4u * capr + (uint32_t)(warp * kRing * 512) +
-                        16u * lane;
-  uint2* tails = reinterpret_cast<uint2*>(wts + capr + kRingFloats);
+  // [a ring of kRing groups a lane for each warp (not with entry weights)]
+  // [per warp its tail: 8-byte slots, slot k of lane l at 32 k + l]
+  constexpr int kRingBytes = MODE == MODE_ENTRY ? 0 : kWarps * kRing * 512;
+  const uint32_t ring = (uint32_t)__cvta_generic_to_shared(smem_raw) + (uint32_t)(warp * kRing * 512) + 16u * lane;
+  uint2* tails = reinterpret_cast<uint2*>(smem_raw + kRingBytes);
   uint2* tail = tails + (size_t)warp * (32 * a.tcap) + lane;
   // with inference (SURR 2) the network's normalisation and BF16 weights
   // follow the tails, copied once per CTA (read by every item, they would
@@ -1167,13 +1191,8 @@ __global__ void __launch_bounds__(32 * kWarps, kWarpsPerSM / kWarps) k_clip_warp
     const int4 g4 = __ldg(reinterpret_cast<const int4*>(a.grp) + b);
     const ClassEnds ge{g4.x >> 2, g4.y >> 2, g4.z >> 2, g4.w >> 2};
 
-    if (MODE == MODE_ENTRY) {
-      for (int e = threadIdx.x; e < n; e += 32 * kWarps) {
-        const uint32_t u = __ldg(a.ent + r0 + e);
-        wts[e] = (u & (kZero | kPad)) ? 0.0f : __ldg(a.w + r0 + e);
-      }
-      __syncthreads();
-    }
+    // (MODE_ENTRY) the row's weights, 0 on padding
+    const float* wts = MODE == MODE_ENTRY ? a.w + r0 : nullptr;
 
     for (int f = f0 + warp; f < f1; f += kWarps) {
       // this item's values: entry e of the row at slot r0 + e of the staged frame
@@ -1271,7 +1290,7 @@ __global__ void __launch_bounds__(32 * kWarps, kWarpsPerSM / kWarps) k_clip_warp
           // a step of the replay: the core sums plus the tail inside [Ln, Hn]
           float ts[5], tc[5], th[5], tl[5];
           uint32_t tn;
-          lane_tail_sums<MODE, KAHAN>(tail, wts, m, Ln, Hn, K, ts, tc, tn);
+          lane_tail_sums<MODE, KAHAN>(tail, m, Ln, Hn, K, ts, tc, tn);
           tn = __reduce_add_sync(0xffffffffu, tn);
           stat(3, 1);
           n_set = cn + (float)tn;
@@ -1402,7 +1421,7 @@ __global__ void __launch_bounds__(32 * kWarps, kWarpsPerSM / kWarps) k_clip_warp
       }
       __syncwarp();   // the tail is rewritten by the warp's next frame
     }
-    // the next unit rewrites unit_s and the shared row weights
+    // the next unit rewrites unit_s
     __syncthreads();
   }
   if (SURR == 2 && a.surr_stats && lane == 0) {
@@ -1454,16 +1473,15 @@ long clip_tail_cap(bool weights, int32_t cap, int warps, int surr) {
   return tcap < 5 ? 0 : tcap;   // (no room for a tail: every step runs as a full pass)
 }
 
-// Shared memory of a launch: a row's weights or the warps' rings, and the tails.
-size_t clip_launch_bytes(bool weights, int32_t cap, int warps, long tcap, int surr) {
-  const long head = weights ? 4 * (((long)cap + 3) & ~3L) : (long)warps * kRing * 512;
-  return (size_t)(head + warps * 256 * tcap + (surr == 2 ? kNetBytes : 0));
+// Shared memory of a launch: the warps' rings (not with entry weights) and tails.
+size_t clip_launch_bytes(bool weights, int warps, long tcap, int surr) {
+  return (size_t)(warps * ((weights ? 0 : kRing * 512) + 256 * tcap) + (surr == 2 ? kNetBytes : 0));
 }
 
 template <int MODE, int PREC, int kWarps, int SURR>
 cudaError_t launch_warp_t(ClipArgs a, int n_ctas, long tcap, int mode, cudaStream_t s) {
   a.tcap = (int32_t)tcap;
-  const size_t smem = clip_launch_bytes(MODE == MODE_ENTRY, a.cap, kWarps, tcap, SURR);
+  const size_t smem = clip_launch_bytes(MODE == MODE_ENTRY, kWarps, tcap, SURR);
   auto k = k_clip_warp<MODE, PREC, kWarps, SURR>;
   // resident CTAs per multiprocessor of this instance at this shared-memory
   // size, cached per device (the first query comes before any capture: the
@@ -1523,7 +1541,7 @@ cudaError_t launch_tail_b(const ClipArgs& a, int n_ctas, int tpb, int mode, cuda
   int warps = tpb == 32 || tpb == 64 || tpb == 128 ? tpb / 32 : 8;
   const long tcap = clip_tail_cap(MODE == MODE_ENTRY, a.cap, warps, SURR);
   // the widest block up to the plan's whose rings and tails fit
-  while (warps > 1 && clip_launch_bytes(MODE == MODE_ENTRY, a.cap, warps, tcap, SURR) + kClipStaticSmem > (size_t)smem_optin())
+  while (warps > 1 && clip_launch_bytes(MODE == MODE_ENTRY, warps, tcap, SURR) + kClipStaticSmem > (size_t)smem_optin())
     warps /= 2;
   switch (warps) {
     case 1: return launch_warp_t<MODE, PREC, 1, SURR>(a, n_ctas, tcap, mode, s);
@@ -1550,8 +1568,8 @@ cudaError_t launch_p(const ClipArgs& a, int n_ctas, int tpb, int32_t prec, int m
 }  // namespace
 
 size_t clip_smem_bytes(int32_t cap, bool weighted) {
-  // the shared memory a clip launch cannot do without: the per-entry weights
-  // of the longest row (a tail can shrink to nothing)
+  // the longest row a launch takes with entry weights: its weights beside an
+  // empty tail, which is also what clip_tail_cap gives the tails room for
   size_t smem = weighted ? (size_t)cap * 4 : 0;
   return (smem + 15) & ~(size_t)15;
 }

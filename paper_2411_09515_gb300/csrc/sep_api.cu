@@ -168,8 +168,9 @@ void set_interp(sep::PixArgs& p, const sep_csr* csr, const sep_params* params) {
 }
 
 sep_status check_bin_fits(sep_ctx* ctx, const sep_csr* csr) {
-  // the clip kernel keeps an entry's index inside its row in 16 bits and, with
-  // per-entry weights, the longest row's weights in shared memory
+  // the clip kernel keeps an entry's index inside its row in 16 bits; with
+  // per-entry weights a row's weights and its tails share one budget
+  // (clip_tail_cap), so the longest row has a lower limit
   if (csr->h.max_row >= 65536) {
     char buf[120];
     snprintf(buf, sizeof buf, "largest bin has %d entries; at most 65535 are supported", csr->h.max_row);
