@@ -128,7 +128,7 @@ def setup_workload(F, rank, seed=2024):
 
 def algorithmic_bytes_clip(F, npix, nvalid, nnz, nbins):
     """Minimum DRAM bytes of one staged integrate + clip of F raw frames
-    (k_stage_ring + k_clip_warp): every raw word once (2 B/pixel/frame), the
+    (k_stage + k_clip_warp): every raw word once (2 B/pixel/frame), the
     calibration planes and the matrix once per launch, the per-bin outputs
     (mean, sigma, count, threshold). The staged copy of the values that the
     two kernels exchange is an implementation choice and is not charged."""
@@ -190,7 +190,7 @@ def source_fingerprint(names=CLIP_SOURCES):
 
 
 def measured_traffic(F):
-    """DRAM bytes (read + write) of k_stage_ring + k_clip_warp per launch of F
+    """DRAM bytes (read + write) of k_stage + k_clip_warp per launch of F
     frames, from the ncu capture recorded in profiles/roofline_traffic.json,
     scaled from its frame count; None when absent or when the kernels' code
     changed since the capture."""
@@ -383,7 +383,7 @@ def run_ours(args):
                        "l2": "inputs larger than L2 (4.58 GB/batch), no flush", "parallelism": f"replicas x{world}",
                        "kept_capacity": kcap, "peak_capacity": pcap, "precision": args.precision,
                        "clip_schedule": plan, "autotune_sample_ms": tune_ms},
-            "roofline": {"bound": "hbm", "kernel": "k_stage_ring + k_clip_warp", "achieved": round(achieved, 1),
+            "roofline": {"bound": "hbm", "kernel": "k_stage + k_clip_warp", "achieved": round(achieved, 1),
                          "peak": peaks.get("hbm_gbs"), "unit": "GB/s",
                          "frac": round(achieved / peaks.get("hbm_gbs"), 4), "traffic": measured_traffic(F),
                          "peak_source": src, "kernel_ms": round(k_ms, 4), "kernel_leg": clip_leg,

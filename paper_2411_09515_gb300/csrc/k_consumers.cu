@@ -90,9 +90,10 @@ int32_t frames_per_thread(int32_t n_frames, int64_t ctas) {
 
 // Four pixels of a warp's 128 (32 apart from i0; VEC: consecutive, one vector
 // access, for float images of a multiple of 4 pixels at an aligned address),
-// for the frames a thread walks: their tables, and their values frame by frame. Pixels past the last
-// read the last one's words, and pixels without a bin take no part in the
-// tests of value(): neither costs the loop over the frames a branch.
+// for the frames a thread walks: their tables, and their values frame by
+// frame. Pixels past the last read the last one's words, and pixels without a
+// bin take no part in the tests of value(): neither costs the loop over the
+// frames a branch.
 template <int DT, bool NORM, bool VEC = false>
 struct PixelColumn {
   static constexpr int kStep = VEC ? 1 : 32;
@@ -596,8 +597,8 @@ __device__ __forceinline__ float valid_value(const PixArgs& p, const void* frame
 // candidates at once as fit the 32 lanes, so all their values are in flight
 // at once instead of one neighbour after another on one lane. The grid fills
 // the GPU whatever the number of frames.
-// 48 Jungfrau-4M frames (90,000 kept pixels each): 145 -> 97 us; 4 frames:
-// 84 -> 22 us.
+// 48 Jungfrau-4M frames (90,000 kept pixels each): 145 -> 92 us; 4 frames:
+// 84 -> 21 us.
 template <int DT, bool NORM>
 __global__ void __launch_bounds__(kPeakThreads) k_peak_flags(PixArgs p, const uint32_t* bitmap, int64_t words,
                                                              const int32_t* idx, const int32_t* n_kept, int64_t kcap,

@@ -62,9 +62,10 @@ constexpr size_t stage_smem_bytes() {
 // The tile's pairs a thread writes: pairs tid + kStageThreads k for
 // k < kScReg stay in registers for every frame, longer lists read the rest at
 // each step (with 7 instead of 8 a 512-frame Jungfrau-4M batch takes 13.3
-// instead of 12.4 ms: its tiles near the beam hold up to 8,000 pairs). loc: the pixel's place in the tile, four consecutive pixels
-// kStageThreads apart (the threads of a warp then store side by side);
-// kTilePix, a NaN, for padding.
+// instead of 12.4 ms: its tiles near the beam hold up to 8,000 pairs). loc:
+// the pixel's place in the tile, four consecutive pixels kStageThreads apart
+// (the threads of a warp then store side by side); kTilePix, a NaN, for
+// padding.
 constexpr int kScReg = 8;
 __device__ __forceinline__ int tile_place(int pix) {
   return pix < 0 ? kTilePix : (pix & 3) * kStageThreads + (pix >> 2);
