@@ -534,7 +534,8 @@ sep_status sep_process_host(sep_ctx* ctx, const sep_csr* csr, const sep_calib* c
  * SEP_DTYPE_U16_JF) or the float32 input, divided by the norm when the
  * matrix has one, for every pixel the matrix uses; pixels it does not use
  * (masked, outside the radial range) receive NaN. These are the values the
- * integration reads. Uses the context's staging buffer. */
+ * integration reads. out_dev may lie over the frames (the call then uses the
+ * context's staging buffer; otherwise no scratch). */
 sep_status sep_correct(sep_ctx* ctx, const sep_csr* csr, const sep_calib* calib, const void* frames_dev,
                        int32_t dtype, int32_t n_frames, float* out_dev, sep_stream stream);
 

@@ -58,7 +58,6 @@ __global__ void k_thresholds(const float* mean, const float* sigma, float k_pick
   if (i < n) thr[i] = __double2float_rd((double)mean[i] + (double)k_pick * (double)sigma[i]);
 }
 
-// One thread per pixel, one warp per bitmap word: every word is written.
 // Level of pixel i in a per-bin profile p (bin level, or the radial
 // interpolation between the bins a and a + 1 with weight t on the upper).
 __device__ __forceinline__ float profile_at(const float* p, int32_t b, const int32_t* ia, const float* it, int64_t i,
@@ -88,6 +87,12 @@ int32_t frames_per_thread(int32_t n_frames, int64_t ctas) {
   return (n_frames + groups - 1) / groups;
 }
 
+// A source of pixel values beside the SEP_DTYPE_*: the batch's staged copy
+// alone, for calls whose outputs may overwrite the frames (a sector a pixel
+// read, against a word of the frame: 1814 against 333 us for 64 corrected raw
+// Jungfrau-4M frames).
+constexpr int kStaged = -1;
+
 // Four pixels of a warp's 128 (32 apart from i0; VEC: consecutive, one vector
 // access, for float images of a multiple of 4 pixels at an aligned address),
 // for the frames a thread walks: their tables, and their values frame by
@@ -100,6 +105,7 @@ struct PixelColumn {
   Level0 cal[kPixPerThread];
   float nm[kPixPerThread];
   uint32_t i[kPixPerThread];   // the pixels, at most npix - 1 (32-bit offsets: one instruction an address)
+  uint32_t at[kPixPerThread];  // kStaged: their slots in a staged row
   bool valid[kPixPerThread];   // inside the image, and with a bin
   __device__ __forceinline__ PixelColumn(const PixArgs& p, int64_t i0) {
 #pragma unroll
@@ -107,6 +113,7 @@ struct PixelColumn {
       i[k] = (uint32_t)min(i0 + kStep * k, p.npix - 1);
       valid[k] = i0 + kStep * k < p.npix && __ldg(p.bop + i[k]) >= 0;
       nm[k] = 1.0f;
+      if (DT == kStaged) at[k] = (uint32_t)max(__ldg(p.pos_of + i[k]), 0);   // (a pixel without a bin has no slot)
       if (DT == SEP_DTYPE_U16_JF) {
         cal[k].set(__ldg(p.ped + i[k]), __ldg(p.gain + i[k]));
         if (!valid[k]) cal[k].limit = 0xffffffffu;
@@ -118,6 +125,11 @@ struct PixelColumn {
     return p.fptr ? (const void*)p.fptr[f] : frame_ptr<DT>(p.frames, f, p.npix);
   }
   __device__ __forceinline__ void load(const PixArgs& p, int64_t f, uint32_t (&w)[kPixPerThread]) const {
+    if (DT == kStaged) {
+#pragma unroll
+      for (int k = 0; k < kPixPerThread; ++k) w[k] = __float_as_uint(__ldg(p.stage + f * p.npos + at[k]));
+      return;
+    }
     const void* fr = frame(p, f);
     if (VEC) {
       const uint4 v = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(fr) + i[0]));
@@ -886,13 +898,16 @@ void launch_correct_t(const PixArgs& p, int32_t n_frames, int32_t fpc, dim3 grid
 
 cudaError_t launch_correct(const PixArgs& p, int32_t n_frames, float* out, cudaStream_t s) {
   if (n_frames <= 0 || p.npix <= 0) return cudaSuccess;
-  const bool raw8 = p.dtype == SEP_DTYPE_U16_JF && p.npix % 8 == 0 && (uintptr_t)out % 16 == 0 &&
+  const bool staged = p.stage != nullptr;
+  const bool raw8 = !staged && p.dtype == SEP_DTYPE_U16_JF && p.npix % 8 == 0 && (uintptr_t)out % 16 == 0 &&
                     (uintptr_t)p.frames % 16 == 0;
   const int64_t per = raw8 ? 8 * kImageThreads : kPixPerCta;
   const int64_t ctas = (p.npix + per - 1) / per;
   const int32_t fpc = frames_per_thread(n_frames, ctas);
   dim3 grid((unsigned)ctas, (unsigned)((n_frames + fpc - 1) / fpc));
-  if (raw8) {
+  if (staged) {
+    k_correct<kStaged, false, false><<<grid, kImageThreads, 0, s>>>(p, n_frames, fpc, out);
+  } else if (raw8) {
     if (p.norm) k_correct_raw8<true><<<grid, kImageThreads, 0, s>>>(p, n_frames, fpc, out);
     else k_correct_raw8<false><<<grid, kImageThreads, 0, s>>>(p, n_frames, fpc, out);
   } else if (p.dtype == SEP_DTYPE_U16_JF) {

@@ -54,6 +54,14 @@ int64_t bitmap_words(int64_t npix) {
   return (w + 7) & ~(int64_t)7;   // 32-byte multiple: vector loads per frame stay aligned
 }
 
+// Do the na bytes at a and the nb bytes at b share one?
+bool overlap(const void* a, int64_t na, const void* b, int64_t nb) {
+  const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+  return a && b && x < y + (uintptr_t)nb && y < x + (uintptr_t)na;
+}
+
+int64_t frame_bytes(const sep_csr* csr, int32_t dtype) { return csr->npix * (dtype == SEP_DTYPE_U16_JF ? 2 : 4); }
+
 sep_status ensure_scratch(sep_ctx* ctx, int64_t bitmap_total, int64_t thr_total, int64_t aux_total = 0) {
   if ((size_t)aux_total > ctx->aux_len) {
     if (ctx->d_aux) cudaFree(ctx->d_aux);
@@ -661,19 +669,31 @@ sep_status sep_correct(sep_ctx* ctx, const sep_csr* csr, const sep_calib* calib,
                        int32_t dtype, int32_t n_frames, float* out_dev, sep_stream stream) {
   sep::DeviceGuard device_guard;
   sep::NvtxRange nvtx_range(__func__);
-  sep_params p{};
-  p.n_iter = 0;
-  p.k_clip = 1.0f;
-  p.k_pick = 0.0f;
-  p.patch = 1;
-  p.min_count = 1;
-  p.precision = SEP_PREC_DWORD;
-  sep_status st = check_common(ctx, csr, calib, frames_dev, dtype, n_frames, &p);
+  sep_params params{};
+  params.n_iter = 0;
+  params.k_clip = 1.0f;
+  params.k_pick = 0.0f;
+  params.patch = 1;
+  params.min_count = 1;
+  params.precision = SEP_PREC_DWORD;
+  sep_status st = check_common(ctx, csr, calib, frames_dev, dtype, n_frames, &params);
   if (st != SEP_OK) return st;
   if (n_frames > 0 && !out_dev) return fail(ctx, SEP_ERR_ARG, "NULL output");
   if (n_frames == 0) return SEP_OK;
-  const cudaError_t e =
-      sep::launch_correct(pix_args(csr, calib, frames_dev, dtype), n_frames, out_dev, (cudaStream_t)stream);
+  sep::PixArgs p = pix_args(csr, calib, frames_dev, dtype);
+  cudaStream_t s = (cudaStream_t)stream;
+  cudaError_t e = cudaSuccess;
+  // An output over the frames themselves: the frames are staged whole before
+  // the first value is written (reading and writing in one pass would meet
+  // words that are corrected values already).
+  if (overlap(frames_dev, frame_bytes(csr, dtype) * n_frames, out_dev, csr->npix * 4 * n_frames)) {
+    if ((st = ensure_stage(ctx, stage_stride(csr) * n_frames)) != SEP_OK) return st;
+    e = enqueue_stage(ctx, csr, calib, frames_dev, nullptr, dtype, n_frames, ctx->d_stage, s);
+    p.stage = ctx->d_stage;
+    p.pos_of = csr->d_pos_of;
+    p.npos = stage_stride(csr);
+  }
+  if (e == cudaSuccess) e = sep::launch_correct(p, n_frames, out_dev, s);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "correct launch");
   return SEP_OK;
 }

@@ -208,7 +208,8 @@ cudaError_t launch_veto(int32_t n_frames, const int32_t* n_peaks, int32_t min_pe
 // Rows list[j] of src to rows j of dst, j < *n_pass (row_bytes a multiple of 4).
 cudaError_t launch_compact_rows(int32_t n_frames, const int32_t* list, const int32_t* n_pass, int64_t row_bytes,
                                 const void* src, void* dst, cudaStream_t s);
-// Corrected frames in image order (NaN where a pixel has no bin).
+// Corrected frames in image order (NaN where a pixel has no bin), from the
+// frames, or from their staged copy with p.stage.
 cudaError_t launch_correct(const PixArgs& p, int32_t n_frames, float* out, cudaStream_t s);
 cudaError_t launch_mark(const PixArgs& p, int32_t n_frames, int32_t nbins, const float* thr, uint32_t* bitmap,
                         int64_t words, cudaStream_t s);
