@@ -898,7 +898,7 @@ void launch_correct_t(const PixArgs& p, int32_t n_frames, int32_t fpc, dim3 grid
 
 cudaError_t launch_correct(const PixArgs& p, int32_t n_frames, float* out, cudaStream_t s) {
   if (n_frames <= 0 || p.npix <= 0) return cudaSuccess;
-  const bool staged = p.stage != nullptr;
+  const bool staged = p.stage != nullptr;   // (image order reads the staged copy only where it has to)
   const bool raw8 = !staged && p.dtype == SEP_DTYPE_U16_JF && p.npix % 8 == 0 && (uintptr_t)out % 16 == 0 &&
                     (uintptr_t)p.frames % 16 == 0;
   const int64_t per = raw8 ? 8 * kImageThreads : kPixPerCta;
@@ -929,7 +929,9 @@ cudaError_t launch_mark_t(const PixArgs& p, int32_t n_frames, int32_t nbins, con
   const int32_t fpc = frames_per_thread(n_frames, ctas);
   dim3 grid((unsigned)ctas, (unsigned)((n_frames + fpc - 1) / fpc));
 #define SEP_MARK_ARGS p, n_frames, fpc, nbins, thr, mean, sigma, k_pick, bitmap, words
-  if (p.dtype == SEP_DTYPE_U16_JF) {
+  if (p.staged_only) {
+    k_mark<kStaged, false, INTERP><<<grid, kImageThreads, 0, s>>>(SEP_MARK_ARGS);
+  } else if (p.dtype == SEP_DTYPE_U16_JF) {
     if (p.norm) k_mark<SEP_DTYPE_U16_JF, true, INTERP><<<grid, kImageThreads, 0, s>>>(SEP_MARK_ARGS);
     else k_mark<SEP_DTYPE_U16_JF, false, INTERP><<<grid, kImageThreads, 0, s>>>(SEP_MARK_ARGS);
   } else {
@@ -951,6 +953,10 @@ cudaError_t launch_mark_interp(const PixArgs& p, int32_t n_frames, int32_t nbins
   return launch_mark_t<true>(p, n_frames, nbins, nullptr, mean, sigma, k_pick, bitmap, words, s);
 }
 
+// Type of the kernel instances that read listed pixels' values: those of raw
+// frames read nothing but the staged copy where the call staged the batch.
+static int32_t listed_source(const PixArgs& p) { return p.staged_only ? SEP_DTYPE_U16_JF : p.dtype; }
+
 int32_t compact_tiles(int64_t words) { return (int32_t)((words + kTileWords - 1) / kTileWords); }
 int32_t peak_chunks(int64_t kcap) { return (int32_t)((kcap + kPeakChunk - 1) / kPeakChunk); }
 
@@ -963,7 +969,7 @@ cudaError_t launch_compact(const PixArgs& p, int32_t n_frames, const uint32_t* b
   k_count_bits<<<grid, 256, 0, s>>>(bitmap, words, scratch, nt);
   const bool nrm = p.norm != nullptr;
 #define SEP_EMIT_ARGS p, bitmap, words, scratch, nt, idx, val, cap, n_kept, status
-  if (p.dtype == SEP_DTYPE_U16_JF) {
+  if (listed_source(p) == SEP_DTYPE_U16_JF) {
     if (nrm) k_emit_kept<SEP_DTYPE_U16_JF, true><<<grid, kCompactThreads, 0, s>>>(SEP_EMIT_ARGS);
     else k_emit_kept<SEP_DTYPE_U16_JF, false><<<grid, kCompactThreads, 0, s>>>(SEP_EMIT_ARGS);
   } else {
@@ -1056,7 +1062,7 @@ cudaError_t launch_peaks(const PixArgs& p, int32_t n_frames, int32_t nbins, cons
 #define SEP_PEMIT(DT, NR)                                                              \
   if (itp) k_peak_emit<DT, NR, true><<<g2, kPeakThreads, 0, s>>>(SEP_PEMIT_ARGS);      \
   else k_peak_emit<DT, NR, false><<<g2, kPeakThreads, 0, s>>>(SEP_PEMIT_ARGS)
-  if (p.dtype == SEP_DTYPE_U16_JF) {
+  if (listed_source(p) == SEP_DTYPE_U16_JF) {
     if (nrm) {
       k_peak_flags<SEP_DTYPE_U16_JF, true><<<g1, kPeakThreads, 0, s>>>(SEP_FLAG_ARGS);
       SEP_PEMIT(SEP_DTYPE_U16_JF, true);

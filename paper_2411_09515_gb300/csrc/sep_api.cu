@@ -60,6 +60,19 @@ bool overlap(const void* a, int64_t na, const void* b, int64_t nb) {
   return a && b && x < y + (uintptr_t)nb && y < x + (uintptr_t)na;
 }
 
+// Does an output of a batch or mixed call (n frames in all, bins rows of
+// profiles) share memory with the `bytes` bytes of frames at `frames`?
+bool outputs_over(const void* frames, int64_t bytes, int64_t n, int64_t bins, const float* mean, const float* sigma,
+                  const int32_t* count, const int32_t* idx, const float* val, int64_t kcap, const int32_t* n_kept,
+                  const sep_peak* peaks, int64_t pcap, const int32_t* n_peaks) {
+  const struct { const void* p; int64_t bytes; } out[8] = {
+      {mean, 4 * bins}, {sigma, 4 * bins}, {count, 4 * bins}, {idx, 4 * kcap * n}, {val, 4 * kcap * n},
+      {n_kept, 4 * n}, {peaks, (int64_t)sizeof(sep_peak) * pcap * n}, {n_peaks, 4 * n}};
+  for (const auto& o : out)
+    if (overlap(frames, bytes, o.p, o.bytes)) return true;
+  return false;
+}
+
 int64_t frame_bytes(const sep_csr* csr, int32_t dtype) { return csr->npix * (dtype == SEP_DTYPE_U16_JF ? 2 : 4); }
 
 sep_status ensure_scratch(sep_ctx* ctx, int64_t bitmap_total, int64_t thr_total, int64_t aux_total = 0) {
@@ -910,6 +923,9 @@ sep_status sep_process_batch(sep_ctx* ctx, const sep_csr* csr, const sep_calib* 
     return st;
   if ((st = ensure_stage(ctx, stage_stride(csr) * n_frames)) != SEP_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
+  const bool over = outputs_over(frames_dev, frame_bytes(csr, dtype) * n_frames, n_frames,
+                                 (int64_t)n_frames * csr->h.nbins, mean_dev, sigma_dev, count_dev, idx_dev, val_dev,
+                                 kept_capacity, n_kept_dev, peaks_dev, peak_capacity, n_peaks_dev);
 
   auto enqueue = [&](int mode) -> cudaError_t {
     // the clip kernel marks the kept pixels as each bin's threshold is known;
@@ -922,6 +938,7 @@ sep_status sep_process_batch(sep_ctx* ctx, const sep_csr* csr, const sep_calib* 
     p.stage = ctx->d_stage;
     p.pos_of = csr->d_pos_of;
     p.npos = stage_stride(csr);
+    p.staged_only = over;
     set_interp(p, csr, params);
     cudaError_t e = cudaMemsetAsync(ctx->d_bitmap, 0, (size_t)(words * n_frames) * 4, s);
     if (e == cudaSuccess) e = enqueue_stage(ctx, csr, calib, frames_dev, nullptr, dtype, n_frames, ctx->d_stage, s);
@@ -1393,6 +1410,11 @@ sep_status sep_process_mixed(sep_ctx* ctx, int32_t n_det, sep_csr* const* csrs, 
       pa.stage = stage;
       pa.pos_of = csr->d_pos_of;
       pa.npos = stage_stride(csr);
+      for (int32_t g : members[d])
+        pa.staged_only = pa.staged_only ||
+                         outputs_over(frames[g].frame_dev, frame_bytes(csr, dtype), n_frames, rows[n_frames], mean_dev,
+                                      sigma_dev, count_dev, idx_dev, val_dev, kept_capacity, n_kept_dev, peaks_dev,
+                                      peak_capacity, n_peaks_dev);
       set_interp(pa, csr, params);
       if (e == cudaSuccess) e = cudaMemsetAsync(bm, 0, (size_t)(words[d] * m) * 4, sd);
       uint64_t align = 0;

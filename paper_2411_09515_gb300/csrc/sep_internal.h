@@ -173,6 +173,9 @@ struct PixArgs {           // what the consumers need to recompute a pixel value
   const float* stage = nullptr;
   const int32_t* pos_of = nullptr;   // [npix] staging position, -1 if not staged
   int64_t npos = 0;
+  // an output of the call lies over the frames: once the batch is staged,
+  // values come from the staged copy alone
+  bool staged_only = false;
   // background at the pixel centre interpolated between bin centres (lower
   // bin, weight on the upper bin, per pixel); null: the centre bin's level
   const int32_t* ia = nullptr;

@@ -58,3 +58,64 @@ def test_correct(rows, cols, F, raw, shift, with_norm):
     assert np.array_equal(np.isnan(got), nan)
     assert np.array_equal(got[~nan].view(np.uint32), want[~nan].view(np.uint32))
     sep.close()
+
+
+KEYS = ("mean", "sigma", "count", "idx", "val", "n_kept", "peaks", "n_peaks")
+
+
+def _equal(got, want):
+    for k in KEYS:
+        assert np.array_equal(got[k].view(np.uint32), want[k].view(np.uint32)), k
+
+
+def _zero_tails(o):
+    o = {k: v.cpu().numpy().copy() for k, v in o.items() if k in KEYS}
+    for f, (k, p) in enumerate(zip(o["n_kept"], o["n_peaks"])):
+        o["idx"][f, k:], o["val"][f, k:], o["peaks"][f, p:] = 0, 0, 0
+    return o
+
+
+@pytest.mark.parametrize("smooth", [0, 1])
+@pytest.mark.parametrize("raw,with_norm", [(False, False), (False, True), (True, False)])
+@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("over", ["mean", "sigma", "val", "idx", "peaks"])
+def test_batch(over, mixed, graph, raw, with_norm, smooth):
+    """One output of the whole path in the frames' own memory (in place: the frames' results over the frames)."""
+    F, det = 9, _detector(131, 126)
+    n, kcap, pcap = det.npix, 3000, 600
+    sep, _, norm, cal = _separator(det, raw, with_norm)
+    sep.set_params(interpolate=smooth, k_pick=2.0)
+    rng = np.random.default_rng(5)
+    if raw:
+        words = (cal[0][0] + cal[1][0] * rng.poisson(6, (F, n))).clip(0, 16383).astype(np.uint16).view(np.int16)
+    else:
+        words = (rng.poisson(6, (F, n)) * (norm if with_norm else 1)).astype(np.float32)
+    t = torch.from_numpy(words).cuda()
+    dtype = SEP_DTYPE_U16_JF if raw else SEP_DTYPE_F32
+    stream = torch.cuda.Stream() if graph else None
+
+    def call(frames, o):
+        if mixed:
+            B.sep_process_mixed(sep.ctx, [sep.csr], [sep.calib], [(0, dtype, frames[f]) for f in range(F)], sep.params,
+                                o["mean"], o["sigma"], o["count"], o["idx"], o["val"], kcap, o["n_kept"], o["peaks"],
+                                pcap, o["n_peaks"], int(graph), stream)
+        else:
+            B.sep_process_batch(sep.ctx, sep.csr, sep.calib, frames, dtype, F, sep.params, o["mean"], o["sigma"],
+                                o["count"], o["idx"], o["val"], kcap, o["n_kept"], o["peaks"], pcap, o["n_peaks"],
+                                int(graph), stream)
+        torch.cuda.synchronize()
+        assert sep.device_status() == 0
+        return _zero_tails(o)
+
+    want = call(t, sep.alloc_outputs(F, kcap, pcap))
+    assert want["n_kept"].min() > 0 and want["n_peaks"].min() > 0
+    for _ in range(2):   # (the second call replays the graph)
+        frames = t.clone()
+        o = sep.alloc_outputs(F, kcap, pcap)
+        size = o[over].numel() * 4
+        assert size <= frames.numel() * frames.element_size()
+        o[over] = frames.view(-1).view(torch.uint8)[:size].view(o[over].dtype).view(o[over].shape)
+        torch.cuda.synchronize()
+        _equal(call(frames, o), want)
+    sep.close()
