@@ -105,7 +105,6 @@ struct PixelColumn {
   Level0 cal[kPixPerThread];
   float nm[kPixPerThread];
   uint32_t i[kPixPerThread];   // the pixels, at most npix - 1 (32-bit offsets: one instruction an address)
-  uint32_t at[kPixPerThread];  // kStaged: their slots in a staged row
   bool valid[kPixPerThread];   // inside the image, and with a bin
   __device__ __forceinline__ PixelColumn(const PixArgs& p, int64_t i0) {
 #pragma unroll
@@ -113,7 +112,6 @@ struct PixelColumn {
       i[k] = (uint32_t)min(i0 + kStep * k, p.npix - 1);
       valid[k] = i0 + kStep * k < p.npix && __ldg(p.bop + i[k]) >= 0;
       nm[k] = 1.0f;
-      if (DT == kStaged) at[k] = (uint32_t)max(__ldg(p.pos_of + i[k]), 0);   // (a pixel without a bin has no slot)
       if (DT == SEP_DTYPE_U16_JF) {
         cal[k].set(__ldg(p.ped + i[k]), __ldg(p.gain + i[k]));
         if (!valid[k]) cal[k].limit = 0xffffffffu;
@@ -125,11 +123,6 @@ struct PixelColumn {
     return p.fptr ? (const void*)p.fptr[f] : frame_ptr<DT>(p.frames, f, p.npix);
   }
   __device__ __forceinline__ void load(const PixArgs& p, int64_t f, uint32_t (&w)[kPixPerThread]) const {
-    if (DT == kStaged) {
-#pragma unroll
-      for (int k = 0; k < kPixPerThread; ++k) w[k] = __float_as_uint(__ldg(p.stage + f * p.npos + at[k]));
-      return;
-    }
     const void* fr = frame(p, f);
     if (VEC) {
       const uint4 v = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(fr) + i[0]));
@@ -169,6 +162,31 @@ struct PixelColumn {
       float x[kPixPerThread];
       values(p, f, w, x);
       if (f + 1 < f1) load(p, f + 1, w);
+      fn(f, x);
+    }
+  }
+};
+
+// The same from the staged copy.
+template <>
+struct PixelColumn<kStaged, false, false> {
+  uint32_t i[kPixPerThread], slot[kPixPerThread];
+  bool valid[kPixPerThread];
+  __device__ __forceinline__ PixelColumn(const PixArgs& p, int64_t i0) {
+#pragma unroll
+    for (int k = 0; k < kPixPerThread; ++k) {
+      i[k] = (uint32_t)min(i0 + 32 * k, p.npix - 1);
+      const int32_t q = __ldg(p.pos_of + i[k]);
+      valid[k] = i0 + 32 * k < p.npix && q >= 0;
+      slot[k] = (uint32_t)max(q, 0);
+    }
+  }
+  template <class F>
+  __device__ __forceinline__ void walk(const PixArgs& p, int32_t f0, int32_t f1, F&& fn) const {
+    for (int32_t f = f0; f < f1; ++f) {
+      float x[kPixPerThread];
+#pragma unroll
+      for (int k = 0; k < kPixPerThread; ++k) x[k] = __ldg(p.stage + f * p.npos + slot[k]);
       fn(f, x);
     }
   }

@@ -159,6 +159,9 @@ struct PixArgs {           // what the consumers need to recompute a pixel value
   const void* frames;
   int64_t npix;
   int32_t rows, cols, dtype;
+  // an output of the call lies over the frames: once the batch is staged,
+  // values come from the staged copy alone
+  bool staged_only = false;
   const float* ped;
   const float* gain;
   const float* norm;       // may be null
@@ -173,9 +176,6 @@ struct PixArgs {           // what the consumers need to recompute a pixel value
   const float* stage = nullptr;
   const int32_t* pos_of = nullptr;   // [npix] staging position, -1 if not staged
   int64_t npos = 0;
-  // an output of the call lies over the frames: once the batch is staged,
-  // values come from the staged copy alone
-  bool staged_only = false;
   // background at the pixel centre interpolated between bin centres (lower
   // bin, weight on the upper bin, per pixel); null: the centre bin's level
   const int32_t* ia = nullptr;
