@@ -109,8 +109,8 @@ def test_every_kept_pixel_a_peak(rows, cols, F):
             assert torch.equal(rec[:, 0].long(), i) and bool((rec[:, 5] == 1).all())
             # one pixel: I is its value, the centroid its centre (a product and a quotient: two roundings)
             assert torch.equal(v[:, 3], frames[f, i])
-            assert torch.allclose(v[:, 1].double(), (i // cols) + 0.5, rtol=2.0 ** -22, atol=0)
-            assert torch.allclose(v[:, 2].double(), (i % cols) + 0.5, rtol=2.0 ** -22, atol=0)
+            assert torch.allclose(v[:, 1].double(), (i // cols).double() + 0.5, rtol=2.0 ** -22, atol=0)
+            assert torch.allclose(v[:, 2].double(), (i % cols).double() + 0.5, rtol=2.0 ** -22, atol=0)
         assert (sep.device_status() != 0) == (n_kept.max() > pcap)
     sep.close()
 
