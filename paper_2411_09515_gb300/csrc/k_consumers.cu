@@ -627,6 +627,7 @@ __global__ void k_scatter_list(const int32_t* idx, const int32_t* n_kept, int64_
 constexpr int kPeakThreads = 256;
 constexpr int kPeakChunk = 256;          // kept entries per flag chunk (8 flag words)
 constexpr int kPeakList = 2048;          // peaks a record CTA lists in shared memory at once
+constexpr int kPeakSlices = 8;           // slices of a frame's records at least
 constexpr int kPeakCtas = 152 * 8;       // CTAs wanted of either peak kernel (8 of 256 threads fit a multiprocessor)
 
 // Bits [j, j + w) of a frame's bitmap, w <= 15 (a second word is read only
@@ -1069,10 +1070,12 @@ cudaError_t launch_peaks(const PixArgs& p, int32_t n_frames, int32_t nbins, cons
   uint32_t* flags = reinterpret_cast<uint32_t*>(scratch);
   int32_t* cnt = scratch + (int64_t)n_frames * nch * 8;
   // either grid: kPeakCtas CTAs over the frames where the lists can use them
-  // (a chunk each in phase 1, a slice of at least 8 chunks each in phase 2)
+  // (a chunk each in phase 1, a slice of at least 8 chunks each in phase 2,
+  // where a frame gets 8 slices even if the frames alone fill the GPU: a
+  // slice's records are a chain of gathers a thread)
   const int32_t want = std::max(1, (kPeakCtas + n_frames - 1) / n_frames);
   dim3 g1((unsigned)std::min(std::max(nch, 1), std::max(want, 64)), (unsigned)n_frames);
-  dim3 g2((unsigned)std::min((nch + 7) / 8 + (nch == 0), std::max(want / 4, 1)), (unsigned)n_frames);
+  dim3 g2((unsigned)std::min((nch + 7) / 8 + (nch == 0), std::max(want / 4, kPeakSlices)), (unsigned)n_frames);
   const bool nrm = p.norm != nullptr;
   const bool itp = p.ia != nullptr && p.it != nullptr;
 #define SEP_FLAG_ARGS p, bitmap, words, idx, n_kept, kcap, patch, min_count, flags, cnt, nch

@@ -1,0 +1,65 @@
+"""Calls that must not fall far behind their ordinary form: each times a call on
+inputs that once sent it to a slow path against the same call on usual inputs,
+in one process on one GPU (best of several, so that other work on the host does
+not count). The limits lie between the ratio with the slow path and without."""
+import numpy as np
+import pytest
+
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2411_09515_gb300 import Separator  # noqa: E402
+
+
+def _best(*calls, rounds=12, repeat=10):
+    """Shortest time of `repeat` runs of each call, the calls taken in turn."""
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    best = [np.inf] * len(calls)
+    for r in range(rounds):
+        for k, call in enumerate(calls):
+            a.record()
+            for _ in range(repeat):
+                call()
+            b.record()
+            torch.cuda.synchronize()
+            if r > 1:
+                best[k] = min(best[k], a.elapsed_time(b))
+    return best
+
+
+def _detector(rows, cols, nbins=500):
+    return synth.Detector("t", rows, cols, dist_m=0.1, center_px=(0.45 * cols, 0.55 * rows), nbins=nbins, split=1)
+
+
+def test_records_of_a_large_batch():
+    """Peak records (a call's time less that of the same call without room for any) of 512 frames with a few
+    hundred peaks among many kept pixels each, against eight calls of 64."""
+    det, F = _detector(1024, 1024, 200), 512
+    sep = Separator.from_detector(det, k_pick=1.0, patch=3, min_count=4)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(4)
+    # one pixel in twelve kept, and a few hundred full 3 x 3 spots
+    frames = torch.empty((F, det.npix), device="cuda")
+    for f in range(F):
+        frames[f] = 2 * (torch.rand(det.npix, generator=g, device="cuda") < 1 / 12)
+        at = torch.randint(2000, det.npix - 2000, (500,), generator=g, device="cuda")
+        for r in (-1024, 0, 1024):
+            for c in (-1, 0, 1):
+                frames[f, at + r + c] = 5.0 - abs(r) / 1024 - 0.5 * abs(c)
+    m = torch.zeros((F, sep.nbins), dtype=torch.float32, device="cuda")
+    s = torch.ones_like(m)
+    k = sep.sparsify(frames, m, s, 1 << 17)
+
+    def peaks(f0, f1, room):
+        sep.peakfind(frames[f0:f1], m[f0:f1], s[f0:f1], k["idx"][f0:f1], k["n_kept"][f0:f1], room)
+
+    def parts(room):
+        for f in range(0, F, 64):
+            peaks(f, f + 64, room)
+
+    full, none, parts_full, parts_none = _best(lambda: peaks(0, F, 4096), lambda: peaks(0, F, 0),
+                                               lambda: parts(4096), lambda: parts(0), rounds=8, repeat=4)
+    assert full - none < 1.0 * (parts_full - parts_none), ((full - none), (parts_full - parts_none))
+    sep.close()
