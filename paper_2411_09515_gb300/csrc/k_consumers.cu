@@ -627,6 +627,7 @@ __global__ void k_scatter_list(const int32_t* idx, const int32_t* n_kept, int64_
 constexpr int kPeakThreads = 256;
 constexpr int kPeakChunk = 256;          // kept entries per flag chunk (8 flag words)
 constexpr int kPeakList = 2048;          // peaks a record CTA lists in shared memory at once
+constexpr int kOwnTest = 4;              // (see k_peak_flags)
 constexpr int kPeakSlices = 8;           // slices of a frame's records at least
 constexpr int kPeakCtas = 152 * 8;       // CTAs wanted of either peak kernel (8 of 256 threads fit a multiprocessor)
 
@@ -660,20 +661,26 @@ __device__ __forceinline__ float valid_value(const PixArgs& p, const void* frame
 //
 // The kernel is bound by the latency of dependent gathers. A thread counts
 // its pixel's kept neighbours a patch row at a time (a run of bitmap bits and
-// a population count); the few entries with enough of them (about 1 in 50)
-// are then tested by the warp together, one lane per patch pixel and as many
-// candidates at once as fit the 32 lanes, so all their values are in flight
-// at once instead of one neighbour after another on one lane. The grid fills
-// the GPU whatever the number of frames.
-// 48 Jungfrau-4M frames (90,000 kept pixels each): 145 -> 92 us; 4 frames:
-// 84 -> 21 us.
+// a population count). Where few entries of a warp have enough of them (about
+// 1 in 50 at the azimuthal model's thresholds), the warp tests them together,
+// one lane per patch pixel and as many candidates at once as fit the 32
+// lanes, so all their values are in flight at once instead of one neighbour
+// after another on one lane. That costs every candidate its whole patch:
+// where its rounds would come to more than 1 / kOwnTest of the patch's pixels
+// (many candidates: low thresholds, large patches with a low min_count), each
+// lane tests its own candidate and stops at the first larger neighbour. The
+// grid fills the GPU whatever the number of frames.
+// 48 raw Jungfrau-4M frames, 90,000 kept pixels each: 145 -> 92 us, 4 frames:
+// 84 -> 21 us. One pixel in six kept (the whole call): 3 x 3 patches 2497 us
+// with every candidate tested by the warp, 1934 with the choice, 5 x 5 10270
+// and 3650, 7 x 7 8300 and 5740; 15 x 15 15.2 ms by the warp, 18.1 ms a lane
+// each. kOwnTest: 2 gives 7820 us for 7 x 7, 8 gives 17.4 ms for 15 x 15.
 template <int DT, bool NORM>
 __global__ void __launch_bounds__(kPeakThreads) k_peak_flags(PixArgs p, const uint32_t* bitmap, int64_t words,
                                                              const int32_t* idx, const int32_t* n_kept, int64_t kcap,
                                                              int32_t patch, int32_t min_count, uint32_t* flags,
                                                              int32_t* chunk_cnt, int32_t n_chunks) {
   __shared__ int32_t cpix_s[kPeakThreads];   // per warp: its candidates' pixels
-  __shared__ int cnt_s[kPeakThreads / 32];
   const int64_t f = blockIdx.y;
   const uint32_t* bm = bitmap + f * words;
   const void* frame = p.fptr ? (const void*)p.fptr[f] : frame_ptr<DT>(p.frames, f, p.npix);
@@ -698,12 +705,27 @@ __global__ void __launch_bounds__(kPeakThreads) k_peak_flags(PixArgs p, const ui
       enough = nk >= min_count;
     }
     const uint32_t em = __ballot_sync(0xffffffffu, enough);
-    uint32_t peaks = 0;
-    if (em) {
-      const int rank = __popc(em & ((1u << lane) - 1u)), nc = __popc(em);
+    const int nc = __popc(em);
+    bool peak = false;
+    if (kOwnTest * ((nc + per - 1) / per) > area) {   // many candidates: each lane its own
+      peak = enough;
+      if (enough) {
+        bool ok;
+        const float vi = valid_value<DT, NORM>(p, frame, f, i, ok);
+        const int cr = i / p.cols, cc = i - cr * p.cols;
+        const int rhi = min(cr + h, p.rows - 1), clo = max(cc - h, 0), chi = min(cc + h, p.cols - 1);
+        for (int r = max(cr - h, 0); r <= rhi && peak; ++r)
+          for (int q = clo; q <= chi && peak; ++q) {
+            const int64_t j = (int64_t)r * p.cols + q;
+            if (j == i) continue;
+            const float vj = valid_value<DT, NORM>(p, frame, f, j, ok);
+            if (ok && !(vi > vj || (vi == vj && i < j))) peak = false;
+          }
+      }
+    } else if (em) {
+      const int rank = __popc(em & ((1u << lane) - 1u));
       if (enough) cand[rank] = i;
       __syncwarp();
-      bool peak = false;
       for (int c0 = 0; c0 < nc; c0 += per) {
         bool fine = true;   // no patch pixel of this lane beats its candidate
         const int sub = per > 1 ? lane / area : 0;
@@ -732,21 +754,12 @@ __global__ void __launch_bounds__(kPeakThreads) k_peak_flags(PixArgs p, const ui
           peak = (b & want) == want;
         }
       }
-      peaks = __ballot_sync(0xffffffffu, peak);
       __syncwarp();   // the list is rewritten by the warp's next chunk
     }
-    if (lane == 0) {
-      flags[f * ((int64_t)n_chunks * 8) + ch * 8 + warp] = peaks;
-      cnt_s[warp] = __popc(peaks);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int c = 0;
-#pragma unroll
-      for (int w8 = 0; w8 < kPeakThreads / 32; ++w8) c += cnt_s[w8];
-      chunk_cnt[f * n_chunks + ch] = c;
-    }
-    __syncthreads();
+    const uint32_t peaks = __ballot_sync(0xffffffffu, peak);
+    if (lane == 0) flags[f * ((int64_t)n_chunks * 8) + ch * 8 + warp] = peaks;
+    const int c = __syncthreads_count(peak);
+    if (threadIdx.x == 0) chunk_cnt[f * n_chunks + ch] = c;
   }
 }
 

@@ -63,3 +63,23 @@ def test_records_of_a_large_batch():
                                                lambda: parts(4096), lambda: parts(0), rounds=8, repeat=4)
     assert full - none < 1.0 * (parts_full - parts_none), ((full - none), (parts_full - parts_none))
     sep.close()
+
+
+def test_peaks_of_many_candidates():
+    """Five by five patches around one pixel in six, against three by three."""
+    det, F = _detector(1500, 1500), 16
+    sep = Separator.from_detector(det, k_pick=1.0)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    frames = torch.randn((F, det.npix), generator=g, device="cuda")
+    m = torch.zeros((F, sep.nbins), dtype=torch.float32, device="cuda")
+    s = torch.ones_like(m)
+    k = sep.sparsify(frames, m, s, det.npix // 4)
+
+    def peaks(patch):
+        sep.set_params(patch=patch, min_count=3)
+        sep.peakfind(frames, m, s, k["idx"], k["n_kept"], det.npix // 16)
+
+    t, t0 = _best(lambda: peaks(5), lambda: peaks(3), rounds=8, repeat=4)
+    assert t < 2.8 * t0, t / t0
+    sep.close()
