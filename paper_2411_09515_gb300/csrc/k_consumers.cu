@@ -353,9 +353,16 @@ __global__ void __launch_bounds__(kImageThreads, 4) k_correct_raw8(PixArgs p, in
 // a tile) left it idle: 48 raw Jungfrau-4M frames 101 -> 97 us, 4 frames 27 ->
 // 25 us, one 16M float frame 20 -> 13 us.
 constexpr int kCompactThreads = 256;
-constexpr int kWordsPerThread = 8;
-constexpr int64_t kTileWords = (int64_t)kCompactThreads * kWordsPerThread;   // bitmap words per CTA
-constexpr int kEmitList = 2048;   // kept pixels a CTA lists in shared memory at once
+constexpr int64_t kTileWords = (int64_t)kCompactThreads * 8;   // bitmap words per CTA
+// ... and tiles of 1024 threads where there are at most kWideCtas: those of a
+// small detector or a few frames do not fill the GPU, and where a threshold
+// keeps most pixels of a tile its threads take them 2048 at a time, round
+// after round (every pixel of one 300 x 301 frame kept: 183 -> 41 us, of one
+// raw Jungfrau-4M frame 227 -> 64, of seven 302 -> 168; few kept: the same).
+// Beyond that the rounds of one tile hide behind other tiles', and the wide
+// tiles are slower where few pixels are kept (40 frames: 306 against 277 us).
+constexpr int kWideThreads = 1024;
+constexpr int64_t kWideCtas = 152 * 4;
 
 // Phase 1 of the ordered compaction: kept pixels per tile of the bitmap.
 __global__ void __launch_bounds__(256) k_count_bits(const uint32_t* bitmap, int64_t words, int32_t* tile_cnt,
@@ -383,12 +390,14 @@ __global__ void __launch_bounds__(256) k_count_bits(const uint32_t* bitmap, int6
 // Phase 2: each CTA writes its tile's kept pixels (ascending) after the
 // pixels of all earlier tiles of the frame; values are recomputed from the
 // frame exactly as the clip kernel computed them.
-template <int DT, bool NORM>
-__global__ void __launch_bounds__(kCompactThreads) k_emit_kept(PixArgs p, const uint32_t* bitmap, int64_t words,
+template <int DT, bool NORM, int NT>
+__global__ void __launch_bounds__(NT) k_emit_kept(PixArgs p, const uint32_t* bitmap, int64_t words,
                                                                const int32_t* tile_cnt, int32_t n_tiles, int32_t* idx,
                                                                float* val, int64_t cap, int32_t* n_kept,
                                                                int32_t* status) {
-  __shared__ int sh[kCompactThreads / 32];
+  constexpr int kWordsPerThread = (int)(kTileWords / NT);
+  constexpr int kEmitList = 8 * NT;   // kept pixels a CTA lists in shared memory at once
+  __shared__ int sh[NT / 32];
   __shared__ int64_t base_s;
   const int64_t f = blockIdx.y;
   const int tile = blockIdx.x;
@@ -419,11 +428,12 @@ __global__ void __launch_bounds__(kCompactThreads) k_emit_kept(PixArgs p, const 
   const int64_t g = p.fidx ? p.fidx[f] : f;   // output row of this frame
   const int64_t w0 = (int64_t)tile * kTileWords + (int64_t)threadIdx.x * kWordsPerThread;
   uint32_t wv[kWordsPerThread];
-  if (w0 + kWordsPerThread <= words) {
+  if (kWordsPerThread == 8 && w0 + kWordsPerThread <= words) {
     const uint4* q = reinterpret_cast<const uint4*>(bm + w0);
     const uint4 a = q[0], b = q[1];
-    wv[0] = a.x; wv[1] = a.y; wv[2] = a.z; wv[3] = a.w;
-    wv[4] = b.x; wv[5] = b.y; wv[6] = b.z; wv[7] = b.w;
+    const uint32_t ab[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int j = 0; j < kWordsPerThread; ++j) wv[j] = ab[j];
   } else {
 #pragma unroll
     for (int j = 0; j < kWordsPerThread; ++j) wv[j] = (w0 + j < words) ? bm[w0 + j] : 0u;
@@ -432,7 +442,7 @@ __global__ void __launch_bounds__(kCompactThreads) k_emit_kept(PixArgs p, const 
 #pragma unroll
   for (int j = 0; j < kWordsPerThread; ++j) cnt += __popc(wv[j]);
   int tile_total;
-  const int first = block_exclusive_scan<kCompactThreads>(cnt, &tile_total, sh);   // this thread's first, in the tile
+  const int first = block_exclusive_scan<NT>(cnt, &tile_total, sh);   // this thread's first, in the tile
   // The tile's kept pixels go through a shared list, kEmitList at a time:
   // each thread lists its own pixels at their ranks, then consecutive
   // threads take consecutive entries, so the value loads of the whole list
@@ -455,7 +465,7 @@ __global__ void __launch_bounds__(kCompactThreads) k_emit_kept(PixArgs p, const 
     }
     __syncthreads();
     const int nr = (int)(n_tile - r0 < kEmitList ? n_tile - r0 : kEmitList);
-    for (int k = threadIdx.x; k < nr; k += kCompactThreads) {
+    for (int k = threadIdx.x; k < nr; k += NT) {
       const int64_t pos = base + r0 + k;
       const int32_t i = lst[k];
       idx[g * cap + pos] = i;
@@ -1001,13 +1011,17 @@ cudaError_t launch_compact(const PixArgs& p, int32_t n_frames, const uint32_t* b
   k_count_bits<<<grid, 256, 0, s>>>(bitmap, words, scratch, nt);
   const bool nrm = p.norm != nullptr;
 #define SEP_EMIT_ARGS p, bitmap, words, scratch, nt, idx, val, cap, n_kept, status
+#define SEP_EMIT(DT, NR)                                                             \
+  if ((int64_t)nt * n_frames <= kWideCtas)                                           \
+    k_emit_kept<DT, NR, kWideThreads><<<grid, kWideThreads, 0, s>>>(SEP_EMIT_ARGS);   \
+  else                                                                                \
+    k_emit_kept<DT, NR, kCompactThreads><<<grid, kCompactThreads, 0, s>>>(SEP_EMIT_ARGS)
   if (listed_source(p) == SEP_DTYPE_U16_JF) {
-    if (nrm) k_emit_kept<SEP_DTYPE_U16_JF, true><<<grid, kCompactThreads, 0, s>>>(SEP_EMIT_ARGS);
-    else k_emit_kept<SEP_DTYPE_U16_JF, false><<<grid, kCompactThreads, 0, s>>>(SEP_EMIT_ARGS);
+    if (nrm) { SEP_EMIT(SEP_DTYPE_U16_JF, true); } else { SEP_EMIT(SEP_DTYPE_U16_JF, false); }
   } else {
-    if (nrm) k_emit_kept<SEP_DTYPE_F32, true><<<grid, kCompactThreads, 0, s>>>(SEP_EMIT_ARGS);
-    else k_emit_kept<SEP_DTYPE_F32, false><<<grid, kCompactThreads, 0, s>>>(SEP_EMIT_ARGS);
+    if (nrm) { SEP_EMIT(SEP_DTYPE_F32, true); } else { SEP_EMIT(SEP_DTYPE_F32, false); }
   }
+#undef SEP_EMIT
 #undef SEP_EMIT_ARGS
   return cudaGetLastError();
 }

@@ -83,3 +83,16 @@ def test_peaks_of_many_candidates():
     t, t0 = _best(lambda: peaks(5), lambda: peaks(3), rounds=8, repeat=4)
     assert t < 2.8 * t0, t / t0
     sep.close()
+
+
+def test_compaction_of_a_full_small_frame():
+    """Every pixel of a few small frames kept, against one in a hundred."""
+    det, F = _detector(300, 301, 60), 7
+    sep = Separator.from_detector(det, k_pick=1.0)
+    full = torch.full((F, det.npix), 2.0, device="cuda")
+    few = full * (torch.arange(det.npix, device="cuda") % 100 == 0)
+    m = torch.zeros((F, sep.nbins), dtype=torch.float32, device="cuda")
+    s = torch.ones_like(m)
+    t, t0 = _best(lambda: sep.sparsify(full, m, s, det.npix), lambda: sep.sparsify(few, m, s, det.npix), repeat=30)
+    assert t < 3 * t0, t / t0
+    sep.close()
