@@ -475,9 +475,20 @@ __global__ void __launch_bounds__(NT) k_emit_kept(PixArgs p, const uint32_t* bit
   }
 }
 
-// Frames a thread walks from which the dense background by bin is better read
-// in columns.
+// Frames a thread walks from which the dense background is better read in
+// columns: by bin without deviates, and interpolated.
 constexpr int32_t kDenseFrames = 8;
+constexpr int32_t kDenseSmoothFrames = 2;
+
+// A pixel's level in a profile with its table in registers (b: its bin, or
+// INTERP the lower one, t the weight on the upper, up: there is one).
+template <bool INTERP>
+__device__ __forceinline__ float profile_level(const float* p, uint32_t b, float t, bool up) {
+  const float lo = __ldg(p + b);
+  if (!INTERP) return lo;
+  const float hi = up ? __ldg(p + b + 1) : 0.0f;
+  return __fadd_rn(__fmul_rn(__fsub_rn(1.0f, t), lo), __fmul_rn(t, hi));
+}
 
 // Densification (Section 3): the background level of every binned pixel
 // (its bin's mean, or RN(mean + RN(sigma z)) with the caller's deviates z;
@@ -537,25 +548,33 @@ __global__ void __launch_bounds__(kImageThreads, NOISE ? 5 : 6) k_dense_backgrou
   }
 }
 
-// The same by bin alone for images of a multiple of 4 pixels at aligned
-// addresses, four consecutive pixels of one frame a thread: with no table but
-// the bins (which stay in the L2) there is little to keep over frames, and one
-// vector access each for bins, deviates and output leaves registers for every
-// warp an SM holds (whole calls with deviates, 64 Jungfrau-4M frames: 542 us
-// against 556 with the kernel above, 7 frames: 79 against 83; without, 7
-// frames: 59 against 64, 16 frames equal, 64 frames 401 against 364).
-template <bool NOISE>
+// The same for images of a multiple of 4 pixels at aligned addresses, four
+// consecutive pixels of one frame a thread, one vector access each for bins,
+// tables, deviates and output, with registers for every warp an SM holds. By
+// bin there is little to keep over frames (whole calls with deviates, 64
+// Jungfrau-4M frames: 542 us against 556 with the kernel above, 7 frames: 79
+// against 83; without, 7 frames: 59 against 64, 16 frames equal, 64 frames
+// 401 against 364); interpolated the tables are worth it from two frames a
+// thread on (one frame: 14.4 us against 22.6, with deviates 18.6 against
+// 25.8; sixteen: 133 against 120, with deviates 193 against 185).
+template <bool NOISE, bool INTERP>
 __global__ void __launch_bounds__(256) k_dense_background_vec(const int32_t* bop, int64_t npix, int32_t nbins,
                                                               const float* mean, const float* sigma,
-                                                              const float* noise, float fill, float* out) {
+                                                              const float* noise, float fill, const int32_t* ia,
+                                                              const float* it, float* out) {
   const int64_t f = blockIdx.y;
   const int64_t i = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
   if (i >= npix) return;
   const int4 b4 = __ldg(reinterpret_cast<const int4*>(bop + i));
-  const int b[4] = {b4.x, b4.y, b4.z, b4.w};
-  float4 z4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  int4 a4 = b4;
+  float4 t4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), z4 = t4;
+  if (INTERP) {
+    a4 = __ldg(reinterpret_cast<const int4*>(ia + i));
+    t4 = __ldg(reinterpret_cast<const float4*>(it + i));
+  }
   if (NOISE) z4 = __ldg(reinterpret_cast<const float4*>(noise + f * npix + i));
-  const float z[4] = {z4.x, z4.y, z4.z, z4.w};
+  const int b[4] = {b4.x, b4.y, b4.z, b4.w}, a[4] = {a4.x, a4.y, a4.z, a4.w};
+  const float t[4] = {t4.x, t4.y, t4.z, t4.w}, z[4] = {z4.x, z4.y, z4.z, z4.w};
   const float* mu = mean + f * nbins;
   const float* sd = NOISE ? sigma + f * nbins : nullptr;
   float x[4];
@@ -563,8 +582,9 @@ __global__ void __launch_bounds__(256) k_dense_background_vec(const int32_t* bop
   for (int k = 0; k < 4; ++k) {
     x[k] = fill;
     if (b[k] >= 0) {
-      x[k] = __ldg(mu + b[k]);
-      if (NOISE) x[k] = __fadd_rn(x[k], __fmul_rn(__ldg(sd + b[k]), z[k]));
+      auto level = [&](const float* p) { return profile_level<INTERP>(p, a[k], t[k], a[k] + 1 < nbins); };
+      x[k] = level(mu);
+      if (NOISE) x[k] = __fadd_rn(x[k], __fmul_rn(level(sd), z[k]));
     }
   }
   *reinterpret_cast<float4*>(out + f * npix + i) = make_float4(x[0], x[1], x[2], x[3]);
@@ -1034,15 +1054,19 @@ cudaError_t launch_densify(const int32_t* bop, int64_t npix, int32_t nbins, int3
   const int64_t ctas = (npix + kPixPerCta - 1) / kPixPerCta;
   const int32_t fpc = frames_per_thread(n_frames, ctas);
   dim3 g1((unsigned)ctas, (unsigned)((n_frames + fpc - 1) / fpc));
-  // by bin: the vector kernel with deviates, and without where the other one
-  // has few frames to hold its bins over
-  const bool vec = !interp_a && npix % 4 == 0 && (uintptr_t)out % 16 == 0 && (uintptr_t)noise % 16 == 0 &&
-                   (noise || fpc < kDenseFrames);
+  // the vector kernel by bin with deviates, and where the other one has few
+  // frames to hold its tables over
+  const bool vec = npix % 4 == 0 && (uintptr_t)out % 16 == 0 && (uintptr_t)noise % 16 == 0 &&
+                   (interp_a ? fpc < kDenseSmoothFrames : noise || fpc < kDenseFrames);
 #define SEP_DENSE_ARGS bop, npix, nbins, n_frames, fpc, mean, sigma, noise, fill, interp_a, interp_t, out
+#define SEP_DENSE_VEC(NZ, IP) \
+  k_dense_background_vec<NZ, IP><<<gv, 256, 0, s>>>(bop, npix, nbins, mean, sigma, noise, fill, interp_a, interp_t, out)
   if (vec) {
     dim3 gv((unsigned)((npix + 1023) / 1024), (unsigned)n_frames);
-    if (noise) k_dense_background_vec<true><<<gv, 256, 0, s>>>(bop, npix, nbins, mean, sigma, noise, fill, out);
-    else k_dense_background_vec<false><<<gv, 256, 0, s>>>(bop, npix, nbins, mean, sigma, noise, fill, out);
+    if (noise && interp_a) SEP_DENSE_VEC(true, true);
+    else if (noise) SEP_DENSE_VEC(true, false);
+    else if (interp_a) SEP_DENSE_VEC(false, true);
+    else SEP_DENSE_VEC(false, false);
   } else if (noise) {
     if (interp_a) k_dense_background<true, true><<<g1, kImageThreads, 0, s>>>(SEP_DENSE_ARGS);
     else k_dense_background<true, false><<<g1, kImageThreads, 0, s>>>(SEP_DENSE_ARGS);
@@ -1050,6 +1074,7 @@ cudaError_t launch_densify(const int32_t* bop, int64_t npix, int32_t nbins, int3
     if (interp_a) k_dense_background<false, true><<<g1, kImageThreads, 0, s>>>(SEP_DENSE_ARGS);
     else k_dense_background<false, false><<<g1, kImageThreads, 0, s>>>(SEP_DENSE_ARGS);
   }
+#undef SEP_DENSE_VEC
 #undef SEP_DENSE_ARGS
   if (cap > 0) {
     dim3 g2((unsigned)std::min<int64_t>((cap + 255) / 256, 64), (unsigned)n_frames);
