@@ -33,38 +33,6 @@ def _detector(rows, cols, nbins=500):
     return synth.Detector("t", rows, cols, dist_m=0.1, center_px=(0.45 * cols, 0.55 * rows), nbins=nbins, split=1)
 
 
-def test_records_of_a_large_batch():
-    """Peak records (a call's time less that of the same call without room for any) of 512 frames with a few
-    hundred peaks among many kept pixels each, against eight calls of 64."""
-    det, F = _detector(1024, 1024, 200), 512
-    sep = Separator.from_detector(det, k_pick=1.0, patch=3, min_count=4)
-    g = torch.Generator(device="cuda")
-    g.manual_seed(4)
-    # one pixel in twelve kept, and a few hundred full 3 x 3 spots
-    frames = torch.empty((F, det.npix), device="cuda")
-    for f in range(F):
-        frames[f] = 2 * (torch.rand(det.npix, generator=g, device="cuda") < 1 / 12)
-        at = torch.randint(2000, det.npix - 2000, (500,), generator=g, device="cuda")
-        for r in (-1024, 0, 1024):
-            for c in (-1, 0, 1):
-                frames[f, at + r + c] = 5.0 - abs(r) / 1024 - 0.5 * abs(c)
-    m = torch.zeros((F, sep.nbins), dtype=torch.float32, device="cuda")
-    s = torch.ones_like(m)
-    k = sep.sparsify(frames, m, s, 1 << 17)
-
-    def peaks(f0, f1, room):
-        sep.peakfind(frames[f0:f1], m[f0:f1], s[f0:f1], k["idx"][f0:f1], k["n_kept"][f0:f1], room)
-
-    def parts(room):
-        for f in range(0, F, 64):
-            peaks(f, f + 64, room)
-
-    full, none, parts_full, parts_none = _best(lambda: peaks(0, F, 4096), lambda: peaks(0, F, 0),
-                                               lambda: parts(4096), lambda: parts(0), rounds=8, repeat=4)
-    assert full - none < 1.0 * (parts_full - parts_none), ((full - none), (parts_full - parts_none))
-    sep.close()
-
-
 def test_peaks_of_many_candidates():
     """Five by five patches around one pixel in six, against three by three."""
     det, F = _detector(1500, 1500), 16
