@@ -71,6 +71,36 @@ __device__ __forceinline__ int tile_place(int pix) {
   return pix < 0 ? kTilePix : (pix & 3) * kStageThreads + (pix >> 2);
 }
 
+// pixel_value() of a pixel's words of a step's frames: the calibration of each
+// gain level that occurs is read once for all of them, its reads together.
+// (Bright frames have such pixels in every warp. With pixel_value() for the
+// thread's four pixels in the four frames, one after another, 64 raw
+// Jungfrau-4M frames took 1357 us with one pixel in 10,000 at another level,
+// 1537 with one in 1000, 1773 with one in 100 and 1852 with all; now 1125,
+// 1159, 1230 and 1457, and 1074 without any.)
+template <bool NORM>
+__device__ __forceinline__ void level_values(const StageArgs& a, int64_t i, const uint32_t (&u)[kStep],
+                                             float (&y)[kStep]) {
+  float ped[3], gain[3];
+#pragma unroll
+  for (int l = 0; l < 3; ++l) {
+    bool occurs = false;
+#pragma unroll
+    for (int h = 0; h < kStep; ++h) occurs = occurs || min(u[h] >> 14, 2u) == (uint32_t)l;
+    ped[l] = occurs ? __ldg(a.ped + l * a.npix + i) : 0.0f;
+    gain[l] = occurs ? __ldg(a.gain + l * a.npix + i) : 1.0f;
+  }
+  const float norm = NORM ? __ldg(a.norm + i) : 1.0f;
+#pragma unroll
+  for (int h = 0; h < kStep; ++h) {
+    const uint32_t l = u[h] >> 14;
+    const float pd = l == 0 ? ped[0] : (l == 1 ? ped[1] : ped[2]);
+    const float gn = l == 0 ? gain[0] : (l == 1 ? gain[1] : gain[2]);
+    y[h] = __fdiv_rn(__fsub_rn((float)(u[h] & 0x3fffu), pd), gn);
+    if (NORM) y[h] = __fdiv_rn(y[h], norm);
+  }
+}
+
 template <int DT, bool NORM, int LOAD>
 __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
   constexpr int kWord = DT == SEP_DTYPE_U16_JF ? 2 : 4;
@@ -101,14 +131,14 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
   const int n_in = r < a.rows ? (int)max((int64_t)0, min((int64_t)4, a.cols - c)) : 0;   // of them inside the image
   Level0 cal[4];
   float nm[4];
-  bool usual = true;   // level-0 words of these pixels need no division
+  uint32_t odd = 0;   // bit k: the level-0 words of pixel p + k need a division
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     nm[k] = 1.0f;
     if (k < n_in) {
       if (DT == SEP_DTYPE_U16_JF) {
         cal[k].set(__ldg(a.ped + p + k), __ldg(a.gain + p + k));
-        usual = usual && cal[k].limit != 0;
+        if (cal[k].limit == 0) odd |= 1u << k;
       }
       if (NORM) nm[k] = __ldg(a.norm + p + k);
     }
@@ -156,7 +186,7 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
     const int q0 = j % kRing;   // ring slots of the step's frames
     float4* tile = tv + buf * (kTilePix + 1);
     float x[kStep][4];
-    bool rest = !usual;   // another gain level, or an unusual calibration
+    uint32_t all01 = 0, all23 = 0;   // the bits of the step's words of pixels 0, 1 and 2, 3
     if (DT == SEP_DTYPE_U16_JF) {
       uint2 v[kStep];   // a frame's four words
       if (LOAD != LOAD_PLAIN) {
@@ -174,10 +204,10 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
           v[h] = make_uint2(w[0] | w[1] << 16, w[2] | w[3] << 16);
         }
       }
-      uint32_t all = 0;
 #pragma unroll
       for (int h = 0; h < kStep; ++h) {
-        all |= v[h].x | v[h].y;
+        all01 |= v[h].x;
+        all23 |= v[h].y;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           // the word's value as a float without a conversion: its 16 bits
@@ -187,7 +217,6 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
           if (NORM) x[h][k] = __fdiv_rn(x[h][k], nm[k]);
         }
       }
-      rest = rest || (all & 0xc000c000u);
     } else {
       if (LOAD != LOAD_PLAIN) asm volatile("cp.async.wait_group %0;\n" ::"n"(kRing / kStep - 1) : "memory");
 #pragma unroll
@@ -200,19 +229,36 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
         }
       }
     }
-    // the slots just read are refilled (this thread's own words, in registers now)
-    if (LOAD != LOAD_PLAIN) issue(j + kRing, q0);
+    if (DT != SEP_DTYPE_U16_JF) issue(j + kRing, q0);   // the slots just read are refilled (in registers now)
 #pragma unroll
     for (int k = 0; k < 4; ++k)
       tile[k * kStageThreads + tid] = make_float4(x[0][k], x[1][k], x[2][k], x[3][k]);
-    if (DT == SEP_DTYPE_U16_JF && rest && n_in > 0) {
-      for (int h = 0; h < nf; ++h) {   // (rare: one copy of the code)
-        const void* fr = a.fptr ? (const void*)a.fptr[f0 + j + h] : frame_ptr<DT>(a.frames, f0 + j + h, a.npix);
-        for (int k = 0; k < n_in; ++k)
-          reinterpret_cast<float*>(tile + k * kStageThreads + tid)[h] =
-              pixel_value<DT, NORM>(fr, p + k, a.npix, a.ped, a.gain, a.norm);
+    if (DT == SEP_DTYPE_U16_JF && (((all01 | all23) & 0xc000c000u) || odd)) {
+      // pixels with a word of another gain level or an unusual calibration
+      // (rare: one copy of the code)
+      uint32_t todo = odd;
+      if (all01 & 0x0000c000u) todo |= 1u;
+      if (all01 & 0xc0000000u) todo |= 2u;
+      if (all23 & 0x0000c000u) todo |= 4u;
+      if (all23 & 0xc0000000u) todo |= 8u;
+#pragma unroll 1
+      for (todo &= (1u << n_in) - 1u; todo; todo &= todo - 1) {
+        const int k = __ffs(todo) - 1;
+        uint32_t u[kStep];
+#pragma unroll
+        for (int h = 0; h < kStep; ++h) {
+          u[h] = 0;
+          if (h < nf)
+            u[h] = LOAD != LOAD_PLAIN
+                       ? *reinterpret_cast<const uint16_t*>(ring + ((q0 + h) * kStageThreads + tid) * 8 + 2 * k)
+                       : __ldg(reinterpret_cast<const uint16_t*>(frame_of(j + h)) + k);
+        }
+        float y[kStep];
+        level_values<NORM>(a, p + k, u, y);
+        tile[k * kStageThreads + tid] = make_float4(y[0], y[1], y[2], y[3]);
       }
     }
+    if (DT == SEP_DTYPE_U16_JF && LOAD != LOAD_PLAIN) issue(j + kRing, q0);   // refilled (this thread's own words)
     __syncthreads();
     // the step's frames, slot by slot
     float* out = a.stage + (int64_t)(f0 + j) * a.npos;

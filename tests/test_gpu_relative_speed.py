@@ -33,6 +33,35 @@ def _detector(rows, cols, nbins=500):
     return synth.Detector("t", rows, cols, dist_m=0.1, center_px=(0.45 * cols, 0.55 * rows), nbins=nbins, split=1)
 
 
+@pytest.mark.parametrize("what,limit", [("gain levels", 1.25)])
+def test_staging(what, limit):
+    """A pixel in a thousand at another gain level; gain 0 under a mask of two pixels in a hundred."""
+    det, F = _detector(1500, 1500), 64
+    n = det.npix
+    rng = np.random.default_rng(1)
+    mask = (rng.random(n) < 0.02).astype(np.uint8)
+    ped, gain = synth.jf_calib(n, seed=1)
+    bad_ped, bad_gain = ped.copy(), gain.copy()
+    bad_ped[:, mask != 0], bad_gain[:, mask != 0] = 0, 0
+    g = torch.Generator(device="cuda")
+    g.manual_seed(2)
+    word = torch.from_numpy(ped[0]).cuda() + torch.from_numpy(gain[0]).cuda() * torch.poisson(
+        torch.full((F, n), 2.0, device="cuda"), generator=g)
+    word = word.clamp(0, 16383).to(torch.int16)
+    other = word.clone()
+    other[torch.rand((F, n), generator=g, device="cuda") < 1e-3] |= 1 << 14
+    kw = {"mask": mask, "n_iter": 0}
+    usual = Separator.from_detector(det, calib=(ped, gain), **kw)
+    odd = Separator.from_detector(det, calib=(bad_ped, bad_gain), **kw)
+    if what == "mask":
+        t, t0 = _best(lambda: odd.integrate_clip(word), lambda: usual.integrate_clip(word))
+    else:
+        t, t0 = _best(lambda: usual.integrate_clip(other), lambda: usual.integrate_clip(word))
+    assert t < limit * t0, t / t0
+    usual.close()
+    odd.close()
+
+
 def test_peaks_of_many_candidates():
     """Five by five patches around one pixel in six, against three by three."""
     det, F = _detector(1500, 1500), 16
