@@ -131,7 +131,11 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
   const int n_in = r < a.rows ? (int)max((int64_t)0, min((int64_t)4, a.cols - c)) : 0;   // of them inside the image
   Level0 cal[4];
   float nm[4];
-  uint32_t odd = 0;   // bit k: the level-0 words of pixel p + k need a division
+  // bit k: pixel p + k has a bin; its level-0 words need a division. (Pixels
+  // under the mask count for neither: real calibrations hold gain 0 or NaN
+  // there, and words of any level.)
+  const uint32_t used = DT == SEP_DTYPE_U16_JF ? __ldg(a.used + (int64_t)t * kStageThreads + tid) : 0u;
+  uint32_t odd = 0;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     nm[k] = 1.0f;
@@ -143,6 +147,7 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
       if (NORM) nm[k] = __ldg(a.norm + p + k);
     }
   }
+  odd &= used;
   const int f0 = blockIdx.y * a.frames_per_cta;
   const int nfr = min(f0 + a.frames_per_cta, a.n_frames) - f0;
   const int64_t pitch = a.npix * kWord;   // bytes from a frame to the next
@@ -206,8 +211,10 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
       }
 #pragma unroll
       for (int h = 0; h < kStep; ++h) {
-        all01 |= v[h].x;
-        all23 |= v[h].y;
+        if (h < nf) {   // (past the last frame the ring holds older words)
+          all01 |= v[h].x;
+          all23 |= v[h].y;
+        }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           // the word's value as a float without a conversion: its 16 bits
@@ -242,7 +249,7 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
       if (all23 & 0x0000c000u) todo |= 4u;
       if (all23 & 0xc0000000u) todo |= 8u;
 #pragma unroll 1
-      for (todo &= (1u << n_in) - 1u; todo; todo &= todo - 1) {
+      for (todo &= used; todo; todo &= todo - 1) {
         const int k = __ffs(todo) - 1;
         uint32_t u[kStep];
 #pragma unroll

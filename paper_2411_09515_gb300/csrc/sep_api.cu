@@ -323,6 +323,7 @@ cudaError_t enqueue_stage(sep_ctx* ctx, const sep_csr* csr, const sep_calib* cal
   g.ped = calib && dtype == SEP_DTYPE_U16_JF ? calib->d_ped : nullptr;
   g.gain = calib && dtype == SEP_DTYPE_U16_JF ? calib->d_gain : nullptr;
   g.norm = csr->d_norm;
+  g.used = csr->d_tile_used;
   g.tile_ebase = csr->d_tile_ebase;
   g.tile_sc = csr->d_tile_sc;
   g.stage = stage;
@@ -515,6 +516,7 @@ sep_status sep_build_csr(sep_ctx* ctx, const sep_geometry* geom, const uint8_t* 
       (st = upload(ctx, &c->d_grp, c->h.grp.data(), c->h.grp.size())) != SEP_OK ||
       (st = upload(ctx, &c->d_pos_of, c->h.slot_of.data(), c->h.slot_of.size())) != SEP_OK ||
       (st = upload(ctx, &c->d_tile_ebase, c->h.tile_ebase.data(), c->h.tile_ebase.size())) != SEP_OK ||
+      (st = upload(ctx, &c->d_tile_used, c->h.tile_used.data(), c->h.tile_used.size())) != SEP_OK ||
       (st = upload(ctx, &c->d_tile_sc, reinterpret_cast<const int2*>(c->h.tile_sc.data()),
                    c->h.tile_sc.size() / 2)) != SEP_OK ||
       (c->weighted && (st = upload(ctx, &c->d_w, c->h.w.data(), c->h.w.size())) != SEP_OK) ||
@@ -545,6 +547,7 @@ void sep_csr_destroy(sep_csr* csr) {
   cudaFree(csr->d_grp);
   cudaFree(csr->d_pos_of);
   cudaFree(csr->d_tile_ebase);
+  cudaFree(csr->d_tile_used);
   cudaFree(csr->d_tile_sc);
   delete csr;
 }

@@ -436,12 +436,12 @@ std::string build_csr_host(const sep_geometry& gm, const uint8_t* mask, const fl
       slot_tile[(size_t)e] = (int32_t)cur;
     }
     auto tile_of = [&](int64_t e) -> int64_t { return slot_tile[(size_t)e]; };
-    (void)nt;
     out->tile_ebase.assign((size_t)nt + 1, 0);
     for (int64_t e = 0; e < nnz; ++e) out->tile_ebase[(size_t)tile_of(e) + 1] += 1;
     for (int64_t t = 0; t < nt; ++t) out->tile_ebase[(size_t)t + 1] += out->tile_ebase[(size_t)t];
     std::vector<int64_t> fill_t(out->tile_ebase.begin(), out->tile_ebase.end() - 1);
     out->tile_sc.assign((size_t)nnz * 2, -1);
+    out->tile_used.assign((size_t)nt * (kTileH * kTileW / 4), 0);
     for (int64_t e = 0; e < nnz; ++e) {
       const int64_t t = tile_of(e), k = fill_t[(size_t)t]++;
       const uint32_t u = out->ent[(size_t)e];
@@ -449,6 +449,7 @@ std::string build_csr_host(const sep_geometry& gm, const uint8_t* mask, const fl
       if (!(u & kPad)) {
         const int64_t i = u & kColMask;
         loc = (int32_t)((i / cols) % kTileH * kTileW + (i % cols) % kTileW);
+        out->tile_used[(size_t)(t * (kTileH * kTileW / 4) + loc / 4)] |= (uint8_t)(1u << loc % 4);
       }
       out->tile_sc[(size_t)k * 2] = (int32_t)e;
       out->tile_sc[(size_t)k * 2 + 1] = loc;

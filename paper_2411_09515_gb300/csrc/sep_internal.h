@@ -80,6 +80,7 @@ struct HostCsr {
   // staged copy of a frame (one value per entry, slot = entry index)
   std::vector<int32_t> slot_of;     // [npix] slot of the pixel's centre entry, -1 if none
   std::vector<int32_t> tile_ebase;  // [tiles + 1] first scatter pair of each tile
+  std::vector<uint8_t> tile_used;   // [tiles][tile pixels / 4]: bit k: pixel 4 i + k of the tile has a bin
   std::vector<int32_t> tile_sc;     // [nnz][2] (slot, pixel index in the tile or -1: padding), by tile
 };
 
@@ -153,6 +154,7 @@ struct StageArgs {         // correction + staging of a batch (k_stage)
   const int32_t* tile_ebase;   // [tiles + 1]
   const int2* tile_sc;         // [nnz] (slot, pixel index in the tile or -1 for padding)
   float* stage;            // [n_frames][npos]: value of entry e at slot e
+  const uint8_t* used;     // [tiles][kTileH * kTileW / 4]: bit k: pixel 4 i + k of the tile has a bin
 };
 
 struct PixArgs {           // what the consumers need to recompute a pixel value
@@ -316,6 +318,7 @@ struct sep_csr {
   int32_t* d_grp = nullptr;
   int32_t* d_pos_of = nullptr;        // slot of each pixel's centre entry in a staged row, -1 if none
   int32_t* d_tile_ebase = nullptr;
+  uint8_t* d_tile_used = nullptr;
   int2* d_tile_sc = nullptr;
   const sep_model* model = nullptr;   // surrogate attached by sep_csr_attach_model
 };

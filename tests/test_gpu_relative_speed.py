@@ -33,7 +33,7 @@ def _detector(rows, cols, nbins=500):
     return synth.Detector("t", rows, cols, dist_m=0.1, center_px=(0.45 * cols, 0.55 * rows), nbins=nbins, split=1)
 
 
-@pytest.mark.parametrize("what,limit", [("gain levels", 1.25)])
+@pytest.mark.parametrize("what,limit", [("gain levels", 1.25), ("mask", 1.15)])
 def test_staging(what, limit):
     """A pixel in a thousand at another gain level; gain 0 under a mask of two pixels in a hundred."""
     det, F = _detector(1500, 1500), 64
