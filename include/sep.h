@@ -510,7 +510,8 @@ sep_status sep_surrogate_train(sep_model* model, const float* x_dev, const float
 sep_status sep_csr_attach_model(sep_csr* csr, const sep_model* model);
 
 /* The whole path from host memory to host memory, pipelined: the batch is
- * cut into chunks of chunk_frames frames (0: 64, a quarter of a smaller batch); chunk c+1 is copied in
+ * cut into chunks of chunk_frames frames (0: a quarter of the batch, at most
+ * 12 frames, but at least 32 MB of frames up to 64); chunk c+1 is copied in
  * while chunk c is processed (sep_process_batch on device buffers owned by
  * the context, three chunk slots) and chunk c-1's results are copied out,
  * on three streams.

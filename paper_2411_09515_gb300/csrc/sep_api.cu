@@ -1037,14 +1037,23 @@ sep_status sep_process_host(sep_ctx* ctx, const sep_csr* csr, const sep_calib* c
   if (n_frames == 0) return SEP_OK;
   const int64_t B = csr->h.nbins, N = csr->npix;
   const size_t px = dtype == SEP_DTYPE_U16_JF ? 2 : 4;
-  // Default chunks: 64 frames, which keep the kernels full, down to a quarter
-  // of a smaller batch, so that its copies overlap its kernels (16 raw
-  // Jungfrau-4M frames as one chunk wait for the whole copy-in before the
-  // first kernel and for the last one before the copy-out), but 32 MB of
-  // frames at least: below that a chunk's launches cost more than they hide.
-  const int64_t quarter = (n_frames + 3) / 4, least = ((int64_t)32 << 20) / (int64_t)(px * N) + 1;
-  const int32_t C = std::min(n_frames, chunk_frames > 0 ? chunk_frames
-                                                        : (int32_t)std::min<int64_t>(std::max(quarter, least), 64));
+  // Default chunks: a quarter of the batch, at most 12 frames, so that copies
+  // overlap kernels (16 raw Jungfrau-4M frames as one chunk wait for the whole
+  // copy-in before the first kernel and for the last one before the copy-out:
+  // 1430 us, in fours 1180), but 32 MB of frames at least (at most 64 frames):
+  // below that a chunk's launches cost more than they hide (300 frames of 256
+  // x 256: 590 us in chunks of 64, 1620 of 12). Chunks of a quarter up to 64
+  // frames left the last copies too long: 100 frames 6.06 ms (5.06 now, 5.88
+  // in chunks of 64), 200 frames 11.2 (9.5, 10.8), 512 frames 24.8 (23.3).
+  const int64_t quarter = std::min<int64_t>(((int64_t)n_frames + 3) / 4, 12);
+  const int64_t least = ((int64_t)32 << 20) / (int64_t)(px * N) + 1;
+  // Outputs over the frames: 64 frames a chunk, which takes a batch of up to
+  // 64 in whole before its first result is copied out.
+  const bool over = outputs_over(frames_host, px * N * n_frames, n_frames, (int64_t)n_frames * B, mean_host, sigma_host,
+                                 count_host, idx_host, val_host, kept_capacity, n_kept_host, peaks_host, peak_capacity,
+                                 n_peaks_host);
+  const int32_t by_default = over ? 64 : (int32_t)std::min<int64_t>(std::max(quarter, least), 64);
+  const int32_t C = std::min(n_frames, chunk_frames > 0 ? chunk_frames : by_default);
   // one slot: frames, mean, sigma, count, idx, val, n_kept, peaks, n_peaks (256-byte aligned pieces)
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const size_t sz[9] = {al(px * N * C), al(4 * B * C), al(4 * B * C), al(4 * B * C), al(4 * kept_capacity * C),

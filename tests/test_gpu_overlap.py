@@ -119,3 +119,26 @@ def test_batch(over, mixed, graph, raw, with_norm, smooth):
         torch.cuda.synchronize()
         _equal(call(frames, o), want)
     sep.close()
+
+
+@pytest.mark.parametrize("F", [16, 64])
+@pytest.mark.parametrize("over", ["idx", "val", "peaks"])
+def test_host_batch(over, F):
+    """Results of a batch of one chunk over its own host frames."""
+    det = _detector(800, 811)   # (2.6 MB a frame: default chunks of less than 16 frames)
+    n, kcap, pcap = det.npix, 40000, 4000
+    sep, _, _, _ = _separator(det, False, False)
+    words = torch.from_numpy(np.random.default_rng(6).poisson(6, (F, n)).astype(np.float32)).pin_memory()
+    ref = sep.process_host(words, sep.alloc_host_outputs(F, kcap, pcap), kcap, pcap)
+    torch.cuda.synchronize()
+    want = _zero_tails(ref)
+    frames = words.clone().pin_memory()
+    o = sep.alloc_host_outputs(F, kcap, pcap)
+    flat = frames.view(-1).view(torch.uint8)
+    size = o[over].numel() * 4
+    # the last words: the frames that are copied in last
+    o[over] = flat[flat.numel() - size:].view(o[over].dtype).view(o[over].shape)
+    sep.process_host(frames, o, kcap, pcap)
+    torch.cuda.synchronize()
+    _equal(_zero_tails(o), want)
+    sep.close()
