@@ -284,10 +284,28 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
         const int2 sc = __ldg(a.tile_sc + eb + q);
         put((uint32_t)sc.x, tile[tile_place(sc.y)]);
       }
+    } else if (DT == SEP_DTYPE_F32) {
+      // the last step of a group, from the same registers (with the list read
+      // again for every pair, two raw Jungfrau-4M frames staged and clipped
+      // without steps took 106 us, three 142; now 86 and 110)
+      auto put = [&](uint32_t q, const float4& v) {
+        float* o = out + q;
+        *o = v.x;
+        if (nf > 1) o[a.npos] = v.y;
+        if (nf > 2) o[2 * a.npos] = v.z;
+      };
+#pragma unroll
+      for (int k = 0; k < kScReg; ++k)
+        if (tid + kStageThreads * k < ne) put(slot[k], tile[loc[k]]);
+#pragma unroll 1
+      for (int q = tid + kStageThreads * kScReg; q < ne; q += kStageThreads) {
+        const int2 sc = __ldg(a.tile_sc + eb + q);
+        put((uint32_t)sc.x, tile[tile_place(sc.y)]);
+      }
     } else {
-      // the last step of a group, a frame at a time from the same registers
-      // (with the list read again for every pair, two raw Jungfrau-4M frames
-      // staged and clipped without steps took 106 us, three 142; now 87 and 105)
+      // (raw frames one after another: the same code spills their registers
+      // in the loop over the full steps; float frames it serves better, three
+      // 16M frames 267 us against 293, 18 mixed frames 589 against 621)
 #pragma unroll 1
       for (int h = 0; h < nf; ++h, out += a.npos) {
         const float* v = reinterpret_cast<const float*>(tile) + h;
