@@ -322,6 +322,72 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
   }
 }
 
+// The same for few frames: two a CTA, by pixel of the tile. There is no step
+// of four frames to fill, nothing to prefetch and no list to hold for later
+// frames, so the CTA is small (512 threads, 33 KB) and three of them hide one
+// another's waits on a multiprocessor, where k_stage keeps one. Bound by that
+// chain of waits (list, words, calibration, write-out). Staging and clip of
+// one raw Jungfrau-4M frame: 71 us (82 by k_stage), two 79 (95); one 1M float
+// frame 27 (31), six 42 (49).
+constexpr int kFewThreads = 512;
+constexpr int kFewFrames = 8;
+constexpr int64_t kFewCtas = 152 * 8;
+
+template <int DT, bool NORM>
+__global__ void __launch_bounds__(kFewThreads, 3) k_stage_few(StageArgs a) {
+  __shared__ float tv[2][kTilePix + 1];   // two frames' values, and a NaN (padding)
+  const int t = blockIdx.x;
+  const int tid = threadIdx.x;
+  const int eb = __ldg(a.tile_ebase + t), ne = __ldg(a.tile_ebase + t + 1) - eb;
+  if (ne == 0) return;
+  if (tid < 2) tv[tid][kTilePix] = __int_as_float(0x7fc00000);
+  const int r0 = t / a.tiles_x * kTileH, c0 = t % a.tiles_x * kTileW;
+  const int f = 2 * blockIdx.y;
+  const bool two = f + 1 < a.n_frames;   // (else the frame's words are read twice)
+  const void* fr[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int g = two ? f + h : f;
+    fr[h] = a.fptr ? (const void*)a.fptr[g] : frame_ptr<DT>(a.frames, g, a.npix);
+  }
+  // (a warp reads 32 pixels side by side, at any alignment)
+#pragma unroll 4
+  for (int k = 0; k < kTilePix / kFewThreads; ++k) {
+    const int pix = tid + kFewThreads * k, r = r0 + pix / kTileW, c = c0 + pix % kTileW;
+    if (r >= a.rows || c >= a.cols) continue;
+    const int64_t p = (int64_t)r * a.cols + c;
+    float x[2];
+    if (DT == SEP_DTYPE_U16_JF) {
+      uint32_t u[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) u[h] = __ldg(reinterpret_cast<const uint16_t*>(fr[h]) + p);
+      const float ped = __ldg(a.ped + p), gain = __ldg(a.gain + p);   // level 0, read beside the words
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (u[h] < 0x4000u) {
+          x[h] = __fdiv_rn(__fsub_rn((float)u[h], ped), gain);
+          if (NORM) x[h] = __fdiv_rn(x[h], __ldg(a.norm + p));
+        } else {
+          x[h] = pixel_value<DT, NORM>(fr[h], p, a.npix, a.ped, a.gain, a.norm);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) x[h] = pixel_value<DT, NORM>(fr[h], p, a.npix, a.ped, a.gain, a.norm);
+    }
+    tv[0][pix] = x[0];
+    if (two) tv[1][pix] = x[1];
+  }
+  __syncthreads();
+  float *o0 = a.stage + (int64_t)f * a.npos, *o1 = o0 + a.npos;
+  for (int q = tid; q < ne; q += kFewThreads) {
+    const int2 sc = __ldg(a.tile_sc + eb + q);
+    const int at = sc.y < 0 ? kTilePix : sc.y;
+    o0[(uint32_t)sc.x] = tv[0][at];
+    if (two) o1[(uint32_t)sc.x] = tv[1][at];
+  }
+}
+
 template <int DT, bool NORM, int LOAD>
 cudaError_t launch_l(const StageArgs& a, dim3 grid, cudaStream_t s) {
   constexpr size_t smem = stage_smem_bytes<DT, LOAD>();
@@ -342,6 +408,14 @@ cudaError_t launch_l(const StageArgs& a, dim3 grid, cudaStream_t s) {
 
 template <int DT, bool NORM>
 cudaError_t launch_v(const StageArgs& a, dim3 grid, cudaStream_t s) {
+  // Few frames: as long as three CTAs a multiprocessor take them in less than
+  // three waves (eight 1M float frames 55 us, k_stage 58; four raw Jungfrau-4M
+  // frames 141 and 131, eight of 1031 x 1065 99 and 97).
+  const dim3 few(grid.x, (unsigned)((a.n_frames + 1) / 2));
+  if (a.n_frames <= kFewFrames && (int64_t)few.x * few.y <= kFewCtas) {
+    k_stage_few<DT, NORM><<<few, kFewThreads, 0, s>>>(a);
+    return cudaGetLastError();
+  }
   // One copy of a thread's four words: every frame at an address aligned to
   // them and the rows' pixels in groups of 4. Copies of 4 bytes: float frames
   // (their words), raw frames of an even width at 4-byte addresses.
@@ -358,9 +432,10 @@ cudaError_t launch_stage(const StageArgs& args, int32_t dtype, bool has_norm, cu
   const int n_tiles = a.tiles_x * a.tiles_y;
   // Frames a CTA: 32, which read the tile's calibration and list once for
   // all, fewer (whole steps) where the grid would hold less than four CTAs a
-  // multiprocessor.
+  // multiprocessor; up to 16 frames all in one where the tiles alone fill the
+  // GPU (ten 1M float frames 76 us, in groups of four 80; sixteen 106 and 112).
   const int64_t share = (int64_t)n_tiles * a.n_frames / (152 * 4) / kStep * kStep;
-  a.frames_per_cta = (int)std::min<int64_t>(std::max<int64_t>(share, kStep), 32);
+  a.frames_per_cta = n_tiles >= 152 && a.n_frames <= 16 ? 16 : (int)std::min<int64_t>(std::max<int64_t>(share, kStep), 32);
   dim3 grid(n_tiles, (a.n_frames + a.frames_per_cta - 1) / a.frames_per_cta);
   if (dtype == SEP_DTYPE_U16_JF)
     return has_norm ? launch_v<SEP_DTYPE_U16_JF, true>(a, grid, s) : launch_v<SEP_DTYPE_U16_JF, false>(a, grid, s);

@@ -38,11 +38,13 @@ def _words(F, n, mask, rng):
     return w
 
 
-# (81 tiles x 67 frames: eight frames a group and a remainder of three; 9 x 1102: eight and six; few frames: one step)
+# (81 tiles x 67 frames: eight frames a group and a remainder of three; 9 x 1102: sixteen and fourteen; up to eight
+# frames: pairs of them a CTA; 169 tiles x 11: one group)
 @pytest.mark.parametrize("with_norm", [False, True])
 @pytest.mark.parametrize("raw", [False, True])
 @pytest.mark.parametrize("rows,cols,F", [(520, 520, 67), (520, 518, 67), (521, 519, 66), (130, 131, 1102), (129, 132, 1),
-                                         (129, 131, 2), (65, 126, 3), (521, 516, 65)])
+                                         (129, 131, 2), (65, 126, 3), (521, 516, 65), (521, 518, 8), (520, 519, 5),
+                                         (129, 130, 9), (830, 831, 11)])
 def test_staged_values_over_steps(rows, cols, F, raw, with_norm):
     rng = np.random.default_rng(rows + cols + F)
     det = synth.Detector("s", rows, cols, dist_m=0.05, center_px=(0.4 * cols, 0.6 * rows), nbins=60, split=2)
