@@ -367,24 +367,24 @@ struct Row {
   const float4* v4;
 };
 
-// Scan of every step-th 16-byte group of [q0, q1) of a row by one lane of a
+// Scan of the 16-byte groups of [q0, q1) of a row by one lane of a
 // warp: fn(v, q) for each of the lane's groups, kLoadsAhead loads issued
 // before their use (groups past q1 are not loaded; fn is not called for
 // them).
 template <class F>
-__device__ __forceinline__ void scan_row(const Row& row, int q0, int q1, int lane, F&& fn, int step = 1) {
-  for (int q = q0 + lane * step; q < q1; q += 32 * step * kLoadsAhead) {
+__device__ __forceinline__ void scan_row(const Row& row, int q0, int q1, int lane, F&& fn) {
+  for (int q = q0 + lane; q < q1; q += 32 * kLoadsAhead) {
     float4 v[kLoadsAhead];
 #pragma unroll
     for (int k = 0; k < kLoadsAhead; ++k)
-      if (q + 32 * step * k < q1) v[k] = __ldg(row.v4 + q + 32 * step * k);
+      if (q + 32 * k < q1) v[k] = __ldg(row.v4 + q + 32 * k);
 #pragma unroll
     for (int k = 0; k < kLoadsAhead; ++k)
-      if (q + 32 * step * k < q1) fn(v[k], q + 32 * step * k);
+      if (q + 32 * k < q1) fn(v[k], q + 32 * k);
   }
 }
 
-// The same with the groups' entry weights: fn(v, w, q). The weights come
+// The same for every step-th group with its entry weights: fn(v, w, q). The weights come
 // through the read-only path like the values (every frame of the bin reads
 // them, so all but the first reads hit the L2 or L1), two pairs at a time (three
 // spill). Held in shared memory beside the tails they left room for 5 to 7

@@ -421,7 +421,7 @@ cudaError_t launch_v(const StageArgs& a, dim3 grid, cudaStream_t s) {
   // (their words), raw frames of an even width at 4-byte addresses.
   if (a.align % (DT == SEP_DTYPE_U16_JF ? 8 : 16) == 0 && a.cols % 4 == 0) return launch_l<DT, NORM, LOAD_VECTOR>(a, grid, s);
   if (DT == SEP_DTYPE_F32 || (a.align % 4 == 0 && a.cols % 2 == 0)) return launch_l<DT, NORM, LOAD_WORD>(a, grid, s);
-  return launch_l<DT, NORM, LOAD_PLAIN>(a, grid, s);
+  return launch_l<DT, NORM, DT == SEP_DTYPE_F32 ? LOAD_WORD : LOAD_PLAIN>(a, grid, s);
 }
 
 }  // namespace

@@ -273,7 +273,6 @@ sep::ClipArgs clip_args(sep_ctx* ctx, const sep_csr* csr, const float* stage, in
   a.bin_list = nullptr;
   a.rowptr = csr->d_rowptr;
   a.grp = csr->d_grp;
-  a.ent = csr->d_ent;
   a.w = csr->d_w;
   a.stage = stage;
   a.cpix = csr->d_cpix;
@@ -508,7 +507,6 @@ sep_status sep_build_csr(sep_ctx* ctx, const sep_geometry* geom, const uint8_t* 
     return cuda_fail(ctx, e, "cudaSetDevice");
   }
   if ((st = upload(ctx, &c->d_rowptr, c->h.rowptr.data(), c->h.rowptr.size())) != SEP_OK ||
-      (st = upload(ctx, &c->d_ent, c->h.ent.data(), c->h.ent.size())) != SEP_OK ||
       (st = upload(ctx, &c->d_cpix, c->h.cpix.data(), c->h.cpix.size())) != SEP_OK ||
       (st = upload(ctx, &c->d_interp_a, c->h.interp_a.data(), c->h.interp_a.size())) != SEP_OK ||
       (st = upload(ctx, &c->d_interp_t, c->h.interp_t.data(), c->h.interp_t.size())) != SEP_OK ||
@@ -537,7 +535,6 @@ void sep_csr_destroy(sep_csr* csr) {
   cudaSetDevice(csr->ctx->device);
   free_plan(csr);
   cudaFree(csr->d_rowptr);
-  cudaFree(csr->d_ent);
   cudaFree(csr->d_cpix);
   cudaFree(csr->d_interp_a);
   cudaFree(csr->d_interp_t);

@@ -99,7 +99,6 @@ struct ClipArgs {
   const int32_t* bin_list; // bins handled by this launch (blockIdx.x indexes it); null = all, in order
   const int32_t* rowptr;
   const int32_t* grp;      // [nbins][4] class ends within a row
-  const uint32_t* ent;     // packed entries: staging position + flags
   const float* w;          // per-entry weight c * norm (NORM variant)
   const float* stage;      // staged values [n_frames][npos] (npos here: the row stride)
   int64_t npos;
@@ -308,7 +307,6 @@ struct sep_csr {
   bool has_norm = false;   // values are divided by a norm (Eq. 1)
   bool weighted = false;   // per-entry weights c * norm (a norm, or exact area fractions)
   int32_t* d_rowptr = nullptr;
-  uint32_t* d_ent = nullptr;
   int32_t* d_cpix = nullptr;          // pixel of each centre entry, else -1
   int32_t* d_interp_a = nullptr;      // radial interpolation of the background (densification)
   float* d_interp_t = nullptr;
