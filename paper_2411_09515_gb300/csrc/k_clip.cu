@@ -1568,8 +1568,8 @@ cudaError_t launch_p(const ClipArgs& a, int n_ctas, int tpb, int32_t prec, int m
 }  // namespace
 
 size_t clip_smem_bytes(int32_t cap, bool weighted) {
-  // the longest row a launch takes with entry weights: its weights beside an
-  // empty tail, which is also what clip_tail_cap gives the tails room for
+  // what clip_tail_cap takes from the tails' budget for a row's entry weights
+  // (read through the caches, they need no shared memory themselves)
   size_t smem = weighted ? (size_t)cap * 4 : 0;
   return (smem + 15) & ~(size_t)15;
 }

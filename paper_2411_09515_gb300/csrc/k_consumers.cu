@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(kImageThreads, 5) k_correct(PixArgs p, int32_t
 // The same for raw frames of a multiple of 8 pixels at 16-byte aligned
 // addresses, eight consecutive pixels a thread: one 16-byte load and two
 // 16-byte stores, and one test of the packed words for another gain level.
-// Bound by memory (64 raw Jungfrau-4M frames: 333 us, 5.5 TB/s of words read
+// Bound by memory (64 raw Jungfrau-4M frames: 333 us, 5.2 TB/s of words read
 // and values written; with four pixels a thread 387 us, bound by the
 // addresses and tests a pixel).
 template <bool NORM>
@@ -801,7 +801,8 @@ __global__ void __launch_bounds__(kPeakThreads) k_peak_flags(PixArgs p, const ui
 // its slice's flagged entries at their ranks in shared memory, kPeakList at a
 // time, and writes the records one peak a thread.
 // 48 Jungfrau-4M frames (750 peaks each): 54 -> 42 us; 4 frames: 55 -> 22 us;
-// one 16M frame: 63 -> 20 us.
+// one 16M frame: 63 -> 20 us. A frame gets at least eight slices: with one each,
+// 512 frames with a min_count of 1 took 7.3 ms in the whole call, now 5.6.
 template <int DT, bool NORM, bool INTERP>
 __global__ void __launch_bounds__(kPeakThreads) k_peak_emit(PixArgs p, int32_t nbins, const float* mean,
                                                             const float* sigma, const uint32_t* bitmap, int64_t words,

@@ -13,7 +13,8 @@
 // buffered, so a step costs one barrier and the warps of a CTA correct the
 // next frames while others still write the last. The raw words of later
 // frames arrive meanwhile in a ring in shared memory (cp.async into the
-// thread's own slots: no registers held, no barrier).
+// thread's own slots: no registers held, no barrier). A call of a few frames
+// takes two of them a CTA instead (k_stage_few).
 //
 // Each value is the same IEEE sequence as pixel_value(): RN32(RN32(adc -
 // pedestal) / gain), then RN32(. / norm); level 0 without a division (Level0).

@@ -190,8 +190,10 @@ void set_interp(sep::PixArgs& p, const sep_csr* csr, const sep_params* params) {
 
 sep_status check_bin_fits(sep_ctx* ctx, const sep_csr* csr) {
   // the clip kernel keeps an entry's index inside its row in 16 bits; with
-  // per-entry weights a row's weights and its tails share one budget
-  // (clip_tail_cap), so the longest row has a lower limit
+  // per-entry weights the tails get what shared memory would leave beside a
+  // row's weights (clip_tail_cap: the number of slots is part of the results,
+  // and stays as it was when the weights were held there), so the longest row
+  // has a lower limit
   if (csr->h.max_row >= 65536) {
     char buf[120];
     snprintf(buf, sizeof buf, "largest bin has %d entries; at most 65535 are supported", csr->h.max_row);
@@ -201,9 +203,10 @@ sep_status check_bin_fits(sep_ctx* ctx, const sep_csr* csr) {
   SEP_CUDA(ctx, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device));
   const size_t need = sep::clip_smem_bytes(csr->h.max_row, csr->weighted) + sep::kClipStaticSmem;
   if (need > (size_t)optin) {
-    char buf[160];
-    snprintf(buf, sizeof buf, "largest bin (%d entries) needs %zu bytes of shared memory, device allows %d",
-             csr->h.max_row, need, optin);
+    char buf[200];
+    snprintf(buf, sizeof buf,
+             "largest bin (%d entries) leaves its tails no room: with entry weights they get what %zu bytes leave of "
+             "the %d bytes of shared memory", csr->h.max_row, need, optin);
     return fail(ctx, SEP_ERR_CSR, buf);
   }
   return SEP_OK;
