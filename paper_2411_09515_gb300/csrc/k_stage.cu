@@ -285,10 +285,10 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
         const int2 sc = __ldg(a.tile_sc + eb + q);
         put((uint32_t)sc.x, tile[tile_place(sc.y)]);
       }
-    } else if (DT == SEP_DTYPE_F32) {
+    } else {
       // the last step of a group, from the same registers (with the list read
       // again for every pair, two raw Jungfrau-4M frames staged and clipped
-      // without steps took 106 us, three 142; now 86 and 110)
+      // without steps took 106 us, three 142; now 86 and 101)
       auto put = [&](uint32_t q, const float4& v) {
         float* o = out + q;
         *o = v.x;
@@ -303,22 +303,7 @@ __global__ void __launch_bounds__(kStageThreads) k_stage(StageArgs a) {
         const int2 sc = __ldg(a.tile_sc + eb + q);
         put((uint32_t)sc.x, tile[tile_place(sc.y)]);
       }
-    } else {
-      // (raw frames one after another: the same code spills their registers
-      // in the loop over the full steps; float frames it serves better, three
-      // 16M frames 267 us against 293, 18 mixed frames 589 against 621)
-#pragma unroll 1
-      for (int h = 0; h < nf; ++h, out += a.npos) {
-        const float* v = reinterpret_cast<const float*>(tile) + h;
-#pragma unroll
-        for (int k = 0; k < kScReg; ++k)
-          if (tid + kStageThreads * k < ne) out[slot[k]] = v[4 * loc[k]];
-#pragma unroll 1
-        for (int q = tid + kStageThreads * kScReg; q < ne; q += kStageThreads) {
-          const int2 sc = __ldg(a.tile_sc + eb + q);
-          out[(uint32_t)sc.x] = v[4 * tile_place(sc.y)];
-        }
-      }
+      return;   // (said here: it frees the registers of the loop over the full steps, which spilled otherwise)
     }
   }
 }
