@@ -379,7 +379,8 @@ sep_status sep_compact_frames(sep_ctx* ctx, int32_t n_frames, const int32_t* fra
  * picking, with the kept-pixel map passed between the steps on the device.
  * Outputs as in the three calls above. The launch sequence is captured once
  * per (csr, calib, dtype, n_frames, capacities, params) into a CUDA graph and
- * replayed on later calls with the same shapes (use_graph = 1).
+ * replayed on later calls with the same shapes (use_graph = 1). An output may
+ * lie over the frames (they are read whole first).
  */
 sep_status sep_process_batch(sep_ctx* ctx, const sep_csr* csr, const sep_calib* calib,
                              const void* frames_dev, int32_t dtype, int32_t n_frames,
